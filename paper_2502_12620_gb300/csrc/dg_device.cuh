@@ -1997,59 +1997,194 @@ __global__ void k_transfer(int nL, int n, const Real* __restrict__ old, Real* __
 }
 
 // ============================================================ conversions
-// modal <-> nodal on arrays shaped [outer][var][mode or point][inner],
-// in place (each thread reads all its values before writing)
+// Modal <-> nodal along one axis of a cell's M values, in place, one line at
+// a time.  P_k(-x) = (-1)^k P_k(x) and the Gauss points are symmetric, so a
+// point pair (q, N-1-q) shares its even and its odd part, and P_0 = 1: 4
+// multiply-adds per line of 3 to nodes and 7 back instead of 9 (2 and 4 of
+// 4 at N = 2, 10 and 12 of 16 at N = 4).  In FP64 the transforms are bound
+// by the multiply-add rate (2 per clock and SM), so that is their time.
+template <int N, typename Real>
+__device__ __forceinline__ void line_to_nodal(const Real (&V)[N][N], Real (&u)[N]) {
+  Real r[N];
+#pragma unroll
+  for (int q = 0; q < N / 2; ++q) {
+    Real e = u[0], o = Real(0);
+#pragma unroll
+    for (int k = 2; k < N; k += 2) e += V[N - 1 - q][k] * u[k];
+#pragma unroll
+    for (int k = 3; k < N; k += 2) o += V[N - 1 - q][k] * u[k];
+    if constexpr (N > 3) {
+      o += V[N - 1 - q][1] * u[1];
+      r[N - 1 - q] = e + o;
+      r[q] = e - o;
+    } else {
+      r[N - 1 - q] = e + V[N - 1 - q][1] * u[1];
+      r[q] = e - V[N - 1 - q][1] * u[1];
+    }
+  }
+  if constexpr (N % 2) {  // the centre point: odd polynomials vanish
+    Real e = u[0];
+#pragma unroll
+    for (int k = 2; k < N; k += 2) e += V[N / 2][k] * u[k];
+    r[N / 2] = e;
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q) u[q] = r[q];
+}
+template <int N, typename Real>
+__device__ __forceinline__ void line_to_modal(const Real (&Vi)[N][N], Real (&u)[N]) {
+  Real s[(N + 1) / 2], d[(N + 1) / 2], r[N];
+#pragma unroll
+  for (int q = 0; q < N / 2; ++q) {
+    s[q] = u[N - 1 - q] + u[q];
+    d[q] = u[N - 1 - q] - u[q];
+  }
+  if constexpr (N % 2) s[N / 2] = u[N / 2];
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    Real acc = Real(0);
+    if (k % 2 == 0) {
+#pragma unroll
+      for (int q = 0; q < (N + 1) / 2; ++q) acc += Vi[k][N - 1 - q] * s[q];
+    } else {
+#pragma unroll
+      for (int q = 0; q < N / 2; ++q) acc += Vi[k][N - 1 - q] * d[q];
+    }
+    r[k] = acc;
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) u[k] = r[k];
+}
+template <int D, int N, bool TO_NODAL, typename Real>
+__device__ __forceinline__ void transform_cell(const Tab<N, Real>& T, Real (&a)[ipow(N, D)]) {
+  constexpr int M = ipow(N, D);
+#pragma unroll
+  for (int ax = 0; ax < D; ++ax) {
+    const int S = ax == 0 ? 1 : ax == 1 ? N : N * N;
+#pragma unroll
+    for (int o = 0; o < M; ++o) {
+      if ((o / S) % N != 0) continue;
+      Real l[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) l[k] = a[o + k * S];
+      if constexpr (TO_NODAL) line_to_nodal<N, Real>(T.V, l);
+      else line_to_modal<N, Real>(T.Vi, l);
+#pragma unroll
+      for (int k = 0; k < N; ++k) a[o + k * S] = l[k];
+    }
+  }
+}
+
+// arrays shaped [outer][var][mode or point][inner], in -> out (which may be
+// in: each thread reads all its values before writing)
 template <int D, int P, typename Real>
-__global__ void k_convert(size_t outer, int inner, Real* __restrict__ X, int to_nodal, Tab<P + 1, Real> T) {
+__global__ void __launch_bounds__(128) k_convert(size_t outer, int inner, const Real* in, Real* out, int to_nodal,
+                                                 Tab<P + 1, Real> T) {
   constexpr int N = P + 1, NV = D + 2, M = ipow(N, D);
   const size_t total = outer * NV * inner;
   const size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= total) return;
   const int c = (int)(w % inner);
   const size_t ov = w / inner;  // outer * NV + v
-  Real* base = X + ov * M * inner + c;
-  Real a[M], t2[M];
+  const Real* src = in + ov * M * inner + c;
+  Real* dst = out + ov * M * inner + c;
+  Real a[M];
 #pragma unroll
-  for (int m = 0; m < M; ++m) a[m] = base[(size_t)m * inner];
-  if (to_nodal) apply_all<D, N, Real>(T.V, a, t2);
-  else apply_all<D, N, Real>(T.Vi, a, t2);
+  for (int m = 0; m < M; ++m) a[m] = src[(size_t)m * inner];
+  if (to_nodal) transform_cell<D, N, true, Real>(T, a);
+  else transform_cell<D, N, false, Real>(T, a);
 #pragma unroll
-  for (int m = 0; m < M; ++m) base[(size_t)m * inner] = a[m];
+  for (int m = 0; m < M; ++m) dst[(size_t)m * inner] = a[m];
+}
+
+// h / sum_i(|u_i| + c) at one point (reading R5); false: not admissible
+template <int D, typename Real>
+__device__ __forceinline__ bool cfl_point(const Real (&u)[D + 2], Real h, Real gamma, Real* best) {
+  const Real ri = Real(1) / u[0];
+  Real ke = Real(0), sv = Real(0);
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    ke += u[1 + j] * u[1 + j];
+    sv += fabs(u[1 + j]) * ri;
+  }
+  const Real p = (gamma - Real(1)) * (u[D + 1] - Real(0.5) * ke * ri);
+  if (!(u[0] > Real(0)) || !(p > Real(0)) || !(p < Real(3.0e38))) return false;
+  const Real v = h / (sv + Real(D) * sqrt(gamma * p * ri));
+  *best = v < *best ? v : *best;
+  return true;
+}
+
+// A modal state into the nodal state buffer, with its CFL minimum: one read
+// and one write of the state, which is what bounds it.  A CTA takes CT
+// consecutive cells, one warp row per variable; the nodal values pass through
+// shared memory to the threads that look at the points.  One atomic per CTA:
+// 4096 blocks at p = 2 took 1.15 ms of conversion and copy and 1.48 ms for
+// the CFL pass (an atomic per warp, all on one address) before.
+template <int D, int P, typename Real>
+struct LoadCfg {
+  static constexpr int NV = D + 2, Q = ipow(P + 1, D);
+  static constexpr int CT = NV * Q * 32 * (int)sizeof(Real) <= 46 * 1024 ? 32 : 16;
+  static constexpr int NT = CT * NV;
+};
+template <int D, int P, typename Real>
+__global__ void __launch_bounds__(LoadCfg<D, P, Real>::NT) k_load_state(
+    size_t cells, int nc, const Real* __restrict__ in, Real* __restrict__ U, const Real* __restrict__ hcell, Real gamma,
+    unsigned long long* lam_bits, int* status, Tab<P + 1, Real> T) {
+  using C = LoadCfg<D, P, Real>;
+  constexpr int N = P + 1, NV = D + 2, Q = ipow(N, D), CT = C::CT;
+  __shared__ Real us[NV][Q][CT];
+  const size_t g0 = (size_t)blockIdx.x * CT;
+  const int lane = threadIdx.x % CT, v = threadIdx.x / CT;
+  const size_t g = g0 + lane;
+  if (g < cells) {
+    const size_t b = g / nc;
+    const size_t off = (b * NV + v) * Q * nc + (g - b * nc);
+    Real a[Q];
+#pragma unroll
+    for (int m = 0; m < Q; ++m) a[m] = __ldcs(&in[off + (size_t)m * nc]);
+    transform_cell<D, N, true, Real>(T, a);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      U[off + (size_t)q * nc] = a[q];
+      us[v][q][lane] = a[q];
+    }
+  }
+  __syncthreads();
+  Real best = Real(3.0e38);
+  bool bad = false;
+  for (int w = threadIdx.x; w < Q * CT; w += C::NT) {
+    const int c = w % CT, q = w / CT;
+    if (g0 + c >= cells) continue;
+    Real x[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) x[k] = us[k][q][c];
+    if (!cfl_point<D, Real>(x, hcell[g0 + c], gamma, &best)) bad = true;
+  }
+  cta_min_atomic<C::NT>((double)best, lam_bits);
+  if (bad) atomicExch(status, kStatusNonFinite);
 }
 
 // ============================================================ CFL kernel
-// dt candidates of the current (nodal) state, used before the first step.
+// dt candidates of the current (nodal) state: CTAs stride over the points
+// (the launch takes a few per SM), one atomic per CTA.
 template <int D, int P, typename Real>
-__global__ void k_cfl(int nL, int n, const Real* __restrict__ U, const Real* __restrict__ hcell,
-                      Real gamma, unsigned long long* lam_bits, int* status) {
+__global__ void __launch_bounds__(256) k_cfl(int nL, int n, const Real* __restrict__ U, const Real* __restrict__ hcell,
+                                             Real gamma, unsigned long long* lam_bits, int* status) {
   constexpr int N = P + 1, NV = D + 2, Q = ipow(N, D);
   const int nc = D == 3 ? n * n * n : n * n;
   const size_t total = (size_t)nL * nc * Q;
-  const size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double best = 3.0e38;
+  Real best = Real(3.0e38);
   bool bad = false;
-  if (w < total) {
+  for (size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x; w < total; w += (size_t)gridDim.x * blockDim.x) {
     const int c = (int)(w % nc);
     const int q = (int)((w / nc) % Q);
     const int b = (int)(w / ((size_t)Q * nc));
     Real u[NV];
+#pragma unroll
     for (int v = 0; v < NV; ++v) u[v] = U[(((size_t)b * NV + v) * Q + q) * nc + c];
-    const Real ri = Real(1) / u[0];
-    Real ke = Real(0), sv = Real(0);
-    for (int j = 0; j < D; ++j) {
-      ke += u[1 + j] * u[1 + j];
-      sv += fabs(u[1 + j]) * ri;
-    }
-    const Real p = (gamma - Real(1)) * (u[D + 1] - Real(0.5) * ke * ri);
-    if (!(u[0] > Real(0)) || !(p > Real(0)) || !(p < Real(3.0e38))) bad = true;
-    else best = (double)(hcell[(size_t)b * nc + c] / (sv + Real(D) * sqrt(gamma * p * ri)));
+    if (!cfl_point<D, Real>(u, hcell[(size_t)b * nc + c], gamma, &best)) bad = true;
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    double u = __shfl_xor_sync(0xffffffffu, best, o);
-    best = u < best ? u : best;
-  }
-  if ((threadIdx.x & 31) == 0 && best < 3.0e38)
-    atomicMin(lam_bits, (unsigned long long)__double_as_longlong(best));
+  cta_min_atomic<256>((double)best, lam_bits);
   if (bad) atomicExch(status, kStatusNonFinite);
 }
 

@@ -1057,13 +1057,34 @@ cudaError_t do_transfer(dgf_forest* f, const RtTransfer& r) {
   return state_f64(f) ? launch_transfer<3, double>(r, f->stream) : launch_transfer<3, float>(r, f->stream);
 }
 
-// modal <-> nodal in place; dbl selects the element type of X
-cudaError_t do_convert(dgf_forest* f, void* X, size_t outer, int inner, int to_nodal, bool dbl) {
+// modal <-> nodal, in -> out (which may be in); dbl selects the element type
+cudaError_t do_convert(dgf_forest* f, const void* in, void* out, size_t outer, int inner, int to_nodal, bool dbl) {
   if (f->d == 2)
-    return dbl ? launch_convert<2, double>(f->p, outer, inner, X, to_nodal, f->tab, f->stream)
-               : launch_convert<2, float>(f->p, outer, inner, X, to_nodal, f->tab, f->stream);
-  return dbl ? launch_convert<3, double>(f->p, outer, inner, X, to_nodal, f->tab, f->stream)
-             : launch_convert<3, float>(f->p, outer, inner, X, to_nodal, f->tab, f->stream);
+    return dbl ? launch_convert<2, double>(f->p, outer, inner, in, out, to_nodal, f->tab, f->stream)
+               : launch_convert<2, float>(f->p, outer, inner, in, out, to_nodal, f->tab, f->stream);
+  return dbl ? launch_convert<3, double>(f->p, outer, inner, in, out, to_nodal, f->tab, f->stream)
+             : launch_convert<3, float>(f->p, outer, inner, in, out, to_nodal, f->tab, f->stream);
+}
+cudaError_t do_load_state(dgf_forest* f, const RtMisc& r) {
+  if (f->d == 2) return state_f64(f) ? launch_load_state<2, double>(r, f->stream) : launch_load_state<2, float>(r, f->stream);
+  return state_f64(f) ? launch_load_state<3, double>(r, f->stream) : launch_load_state<3, float>(r, f->stream);
+}
+
+// device memory of the forest's device (plain or managed)?
+bool on_device(const void* p, int device) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == device;
+}
+
+// A caller's buffer that a kernel may read or write in place of a copy: memory
+// of the forest's device, aligned to its elements.  Anything else a copy can
+// reach (host memory, another device's, unaligned) keeps the staged copy.
+bool kernel_reaches(const dgf_forest* f, const void* p, int is_device, size_t elem) {
+  return is_device && (uintptr_t)p % elem == 0 && on_device(p, f->device);
 }
 
 // compute-precision buffer -> state-precision buffer (compensated form: FP32 -> FP64)
@@ -1560,18 +1581,27 @@ dgf_status dgf_set_state(dgf_forest* f, const void* src, int is_device) {
   if (!src) return fail(DGF_EINVAL, "null source");
   DeviceGuard dg(f->device);
   const size_t bytes = (size_t)f->nL * f->nv * f->M * f->nc * f->sesize;
-  void* U = state_ptr(f);
-  dgf_status st = cuda_check(
-      cudaMemcpyAsync(U, src, bytes, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, f->stream),
-      "set_state");
-  if (st) return st;
-  // a host source is read by the copy engine possibly after the copy call
-  // returns: wait before the caller may release it
-  if (!is_device && (st = cuda_check(cudaStreamSynchronize(f->stream), "set_state"))) return st;
+  dgf_status st;
+  RtMisc r = misc_args(f, 0);
+  if (kernel_reaches(f, src, is_device, f->sesize)) {
+    r.U = src;
+  } else {
+    void* tmp = f->comp ? f->U64[1 - f->cur].ptr : f->U[1].ptr;  // free between time steps
+    st = cuda_check(
+        cudaMemcpyAsync(tmp, src, bytes, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, f->stream),
+        "set_state");
+    if (st) return st;
+    // a host source is read by the copy engine possibly after the copy call
+    // returns: wait before the caller may release it
+    if (!is_device && (st = cuda_check(cudaStreamSynchronize(f->stream), "set_state"))) return st;
+    r.U = tmp;
+  }
   // the device holds values at the Gauss points: u = V K per (leaf, var, cell)
-  if ((st = cuda_check(do_convert(f, U, (size_t)f->nL, f->nc, 1, state_f64(f)), "to nodal"))) return st;
+  k_reset_lam<<<1, 1, 0, f->stream>>>((DevScalars*)f->scal.ptr);
+  if ((st = cuda_check(cudaGetLastError(), "reset"))) return st;
+  if ((st = cuda_check(do_load_state(f, r), "to nodal"))) return st;
   f->have_state = true;
-  return init_lambda(f);
+  return DGF_OK;
 }
 
 dgf_status dgf_get_state(dgf_forest* f, void* dst, int is_device) {
@@ -1580,11 +1610,13 @@ dgf_status dgf_get_state(dgf_forest* f, void* dst, int is_device) {
   if (!f->have_state) return fail(DGF_ESTATE, "no state set");
   DeviceGuard dg(f->device);
   const size_t bytes = (size_t)f->nL * f->nv * f->M * f->nc * f->sesize;
+  if (kernel_reaches(f, dst, is_device, f->sesize)) {
+    dgf_status st = cuda_check(do_convert(f, state_ptr(f), dst, (size_t)f->nL, f->nc, 0, state_f64(f)), "to modal");
+    return st ? st : cuda_check(cudaStreamSynchronize(f->stream), "get_state");
+  }
   void* tmp = f->comp ? f->U64[1 - f->cur].ptr : f->U[1].ptr;  // free between time steps
-  dgf_status st = cuda_check(cudaMemcpyAsync(tmp, state_ptr(f), bytes, cudaMemcpyDeviceToDevice, f->stream),
-                             "get_state");
+  dgf_status st = cuda_check(do_convert(f, state_ptr(f), tmp, (size_t)f->nL, f->nc, 0, state_f64(f)), "to modal");
   if (st) return st;
-  if ((st = cuda_check(do_convert(f, tmp, (size_t)f->nL, f->nc, 0, state_f64(f)), "to modal"))) return st;
   return copy_state(f, dst, tmp, bytes, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
 }
 
@@ -1620,7 +1652,7 @@ dgf_status dgf_fill_guardcells(dgf_forest* f, void* guard, int is_device) {
   if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gmod.ptr, 0)), "guard");
   if (st) return st;
   const bool dbl = f->precision == DGF_FP64;
-  if ((st = cuda_check(do_convert(f, f->gmod.ptr, (size_t)f->nL * 2 * f->d, f->nt, 0, dbl), "to modal"))) return st;
+  if ((st = cuda_check(do_convert(f, f->gmod.ptr, f->gmod.ptr, (size_t)f->nL * 2 * f->d, f->nt, 0, dbl), "to modal"))) return st;
   const void* out = f->gmod.ptr;
   if (f->comp) {
     if (!ensure(f, f->gmod64, count * sizeof(double))) return fail(DGF_ENOMEM, "guard allocation failed");
@@ -1640,7 +1672,7 @@ dgf_status dgf_dg_residual(dgf_forest* f, void* dst, int is_device) {
   if (st) return st;
   if ((st = cuda_check(do_stage(f, stage_args(f, 0, 1, 0.0, 1.0, 1, 0)), "stage"))) return st;
   const bool dbl = f->precision == DGF_FP64;
-  if ((st = cuda_check(do_convert(f, f->U[1].ptr, (size_t)f->nL, f->nc, 0, dbl), "to modal"))) return st;
+  if ((st = cuda_check(do_convert(f, f->U[1].ptr, f->U[1].ptr, (size_t)f->nL, f->nc, 0, dbl), "to modal"))) return st;
   const size_t count = (size_t)f->nL * f->nv * f->M * f->nc;
   const void* out = f->U[1].ptr;
   if (f->comp) {
@@ -2107,17 +2139,6 @@ dgf_status noalloc_scratch(int device, void** out) {
   return DGF_OK;
 }
 
-// device memory of the forest's device (plain or managed)?  Host pointers
-// would reach the kernels and fault there, so they are refused up front.
-bool on_device(const void* p, int device) {
-  cudaPointerAttributes a{};
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == device;
-}
-
 }  // namespace
 
 extern "C" dgf_status dgf_dg_residual_noalloc(dgf_forest* f, const void* U_nodal, void* L_nodal) {
@@ -2128,6 +2149,7 @@ extern "C" dgf_status dgf_dg_residual_noalloc(dgf_forest* f, const void* U_nodal
     return fail(DGF_EINVAL, "state pointers must be 16-byte aligned");
   if (f->comp) return fail(DGF_EUNSUPPORTED, "dgf_dg_residual_noalloc: compensated forests are not supported");
   DeviceGuard dg(f->device);
+  // host pointers would reach the kernels and fault there: refused up front
   if (!on_device(U_nodal, f->device) || !on_device(L_nodal, f->device))
     return fail(DGF_EINVAL, "dgf_dg_residual_noalloc: state pointers must be device memory of the forest's device");
   const size_t need = (size_t)f->nL * 2 * f->d * f->nv * f->NFP * f->nt * f->esize;

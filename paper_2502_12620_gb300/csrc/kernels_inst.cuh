@@ -313,7 +313,8 @@ static cudaError_t cfl_p(const RtMisc& r, cudaStream_t s) {
   const int nc = D == 3 ? r.n * r.n * r.n : r.n * r.n;
   const size_t total = (size_t)r.nL * nc * ipow(P + 1, D);
   const int th = 256;
-  k_cfl<D, P, Real><<<(unsigned)((total + th - 1) / th), th, 0, s>>>(
+  const size_t ctas = (total + th - 1) / th, most = 152 * 8;
+  k_cfl<D, P, Real><<<(unsigned)(ctas < most ? ctas : most), th, 0, s>>>(
       r.nL, r.n, (const Real*)r.U, (const Real*)r.hcell, (Real)r.gamma, r.lam_bits, r.status);
   return cudaGetLastError();
 }
@@ -373,11 +374,24 @@ static cudaError_t transfer_p(const RtTransfer& r, cudaStream_t s) {
 }
 
 template <int D, int P, typename Real>
-static cudaError_t convert_p(size_t outer, int inner, void* X, int to_nodal, const RtTables& T, cudaStream_t s) {
+static cudaError_t convert_p(size_t outer, int inner, const void* in, void* out, int to_nodal, const RtTables& T,
+                             cudaStream_t s) {
   const size_t total = outer * (D + 2) * inner;
   const int th = 128;
-  k_convert<D, P, Real><<<(unsigned)((total + th - 1) / th), th, 0, s>>>(outer, inner, (Real*)X, to_nodal,
-                                                                       make_tab<P + 1, Real>(T));
+  k_convert<D, P, Real><<<(unsigned)((total + th - 1) / th), th, 0, s>>>(outer, inner, (const Real*)in, (Real*)out,
+                                                                       to_nodal, make_tab<P + 1, Real>(T));
+  return cudaGetLastError();
+}
+
+template <int D, int P, typename Real>
+static cudaError_t load_state_p(const RtMisc& r, cudaStream_t s) {
+  using C = LoadCfg<D, P, Real>;
+  const int nc = D == 3 ? r.n * r.n * r.n : r.n * r.n;
+  const size_t cells = (size_t)r.nL * nc;
+  if (cells == 0) return cudaSuccess;
+  k_load_state<D, P, Real><<<(unsigned)((cells + C::CT - 1) / C::CT), C::NT, 0, s>>>(
+      cells, nc, (const Real*)r.U, (Real*)r.Uout, (const Real*)r.hcell, (Real)r.gamma, r.lam_bits, r.status,
+      make_tab<P + 1, Real>(r.T));
   return cudaGetLastError();
 }
 
@@ -576,13 +590,19 @@ static cudaError_t launch_guard_batch_p(const void* members, const int* bstart, 
     DGF_DISPATCH_P(transfer_p, r, s)                                                        \
   }                                                                                         \
   template <>                                                                               \
-  cudaError_t launch_convert<DIM, REAL>(int p, size_t outer, int inner, void* X, int to_nodal, \
+  cudaError_t launch_load_state<DIM, REAL>(const RtMisc& r, cudaStream_t s) {               \
+    constexpr int D = DIM;                                                                  \
+    using Real = REAL;                                                                      \
+    DGF_DISPATCH_P(load_state_p, r, s)                                                      \
+  }                                                                                         \
+  template <>                                                                               \
+  cudaError_t launch_convert<DIM, REAL>(int p, size_t outer, int inner, const void* in, void* out, int to_nodal, \
                                         const RtTables& T, cudaStream_t s) {                \
     switch (p) {                                                                            \
-      case 0: return convert_p<DIM, 0, REAL>(outer, inner, X, to_nodal, T, s);              \
-      case 1: return convert_p<DIM, 1, REAL>(outer, inner, X, to_nodal, T, s);              \
-      case 2: return convert_p<DIM, 2, REAL>(outer, inner, X, to_nodal, T, s);              \
-      case 3: return convert_p<DIM, 3, REAL>(outer, inner, X, to_nodal, T, s);              \
+      case 0: return convert_p<DIM, 0, REAL>(outer, inner, in, out, to_nodal, T, s);        \
+      case 1: return convert_p<DIM, 1, REAL>(outer, inner, in, out, to_nodal, T, s);        \
+      case 2: return convert_p<DIM, 2, REAL>(outer, inner, in, out, to_nodal, T, s);        \
+      case 3: return convert_p<DIM, 3, REAL>(outer, inner, in, out, to_nodal, T, s);        \
     }                                                                                       \
     return cudaErrorInvalidValue;                                                           \
   }                                                                                         \

@@ -126,10 +126,13 @@ template <int D, typename Real>
 cudaError_t launch_limit(const RtMisc& r, cudaStream_t s);
 template <int D, typename Real>
 cudaError_t launch_transfer(const RtTransfer& r, cudaStream_t s);
-// modal <-> nodal in place on [outer][var][mode/point][inner]
+// modal <-> nodal on [outer][var][mode/point][inner], in -> out (in = out allowed)
 template <int D, typename Real>
-cudaError_t launch_convert(int p, size_t outer, int inner, void* X, int to_nodal, const RtTables& T,
-                           cudaStream_t s);
+cudaError_t launch_convert(int p, size_t outer, int inner, const void* in, void* out, int to_nodal,
+                           const RtTables& T, cudaStream_t s);
+// modal state r.U -> nodal state r.Uout with its CFL minimum
+template <int D, typename Real>
+cudaError_t launch_load_state(const RtMisc& r, cudaStream_t s);
 template <int D, typename Real>
 size_t stage_smem_bytes(int p, int n);
 // batches (3D, n_seg 8, FP32, plain form): per-forest argument packing on the
