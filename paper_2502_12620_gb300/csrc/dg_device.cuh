@@ -1818,38 +1818,66 @@ __device__ __forceinline__ Real pressure_root(const Real (&ub)[D + 2], const Rea
 // theta_2 the pressure to >= eps p(ubar) at every volume and face Gauss
 // point; the cell becomes ubar + theta_1 theta_2 (u - ubar) (only written
 // when limited).  A cell whose mean is not admissible sets the status word.
-// One thread per (leaf, cell).
+//
+// One thread per cell, its values read once and kept on chip: in registers
+// where they fit (NV Q <= 40), else in the thread's own column of shared
+// memory.  What bounds it is the instruction count of the Q + 2 D (p+1)^(D-1)
+// check points, so a point costs its traces and the product form of the
+// pressure bound, rho (E - eps_p / (gamma - 1)) >= |m|^2 / 2; only a cell
+// where that or the density bound fails forms theta (from memory, below).
 template <int D, int P, typename Real>
-__global__ void k_limit(int nL, int n, Real* __restrict__ U, const Real* __restrict__ geo,
-                        const unsigned char* __restrict__ affine, Real gamma, Real eps, int* status,
-                        Tab<P + 1, Real> T) {
+struct LimitCfg {
+  static constexpr int NV = D + 2, Q = ipow(P + 1, D);
+  static constexpr bool REGS = NV * Q <= 40;
+  static constexpr int BYTES = NV * Q * (int)sizeof(Real);  // per cell
+  static constexpr int NT = REGS ? 128 : BYTES * 64 <= 47 * 1024 ? 64 : BYTES * 32 <= 47 * 1024 ? 32 : 16;
+};
+template <int D, int P, typename Real>
+__global__ void __launch_bounds__(LimitCfg<D, P, Real>::NT) k_limit(
+    int nL, int lnc, Real* __restrict__ U, const Real* __restrict__ geo, const unsigned char* __restrict__ affine,
+    Real gamma, Real eps, int* status, const __grid_constant__ Tab<P + 1, Real> T) {
+  using C = LimitCfg<D, P, Real>;
   constexpr int N = P + 1, NV = D + 2, Q = ipow(N, D), NFP = ipow(N, D - 1);
   constexpr int NG = ((1 << D) - 1) * D;
-  const int nc = D == 3 ? n * n * n : n * n;
-  const size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= (size_t)nL * nc) return;
-  const int b = (int)(w / nc), c = (int)(w % nc);
-  Real* u = U + (size_t)b * NV * Q * nc + c;
+  const int nc = 1 << lnc;  // n is a power of two
+  const size_t w = (size_t)blockIdx.x * C::NT + threadIdx.x;
+  if (w >> lnc >= (size_t)nL) return;
+  const size_t b = w >> lnc;
+  const int c = (int)(w & (size_t)(nc - 1));
+  Real* u = U + b * NV * Q * nc + c;
   const Real gm1 = gamma - Real(1);
+  Real reg[C::REGS ? NV * Q : 1];
+  __shared__ Real col[C::REGS ? 1 : NV * Q][C::REGS ? 1 : C::NT];
+  auto X = [&](int v, int q) -> Real {
+    if constexpr (C::REGS) return reg[v * Q + q];
+    else return col[v * Q + q][threadIdx.x];
+  };
+#pragma unroll(C::REGS ? NV * Q : 16)
+  for (int i = 0; i < NV * Q; ++i) {
+    if constexpr (C::REGS) reg[i] = u[(size_t)i * nc];
+    else col[i][threadIdx.x] = u[(size_t)i * nc];
+  }
   // J-weighted mean
   Real ub[NV], wsum = Real(0);
 #pragma unroll
   for (int v = 0; v < NV; ++v) ub[v] = Real(0);
   const bool aff = affine[b] != 0;
+#pragma unroll(C::REGS ? Q : 3)
   for (int q = 0; q < Q; ++q) {
     Real xi[D], wq = Real(1);
+#pragma unroll
     for (int a = 0, r = q; a < D; ++a, r /= N) {
       xi[a] = T.x[r % N];
       wq *= T.w[r % N];
     }
     if (!aff) {
       Real t[D][D];
-      tangents<D, Real>(geo + (size_t)b * NG * nc + c, nc, xi, t);
+      tangents<D, Real>(geo + b * NG * nc + c, nc, xi, t);
       wq *= jacobian_det<D, Real>(t);
     }
     wsum += wq;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) ub[v] += wq * u[((size_t)v * Q + q) * nc];
+    for (int v = 0; v < NV; ++v) ub[v] += wq * X(v, q);
   }
 #pragma unroll
   for (int v = 0; v < NV; ++v) ub[v] /= wsum;
@@ -1858,11 +1886,44 @@ __global__ void k_limit(int nL, int n, Real* __restrict__ U, const Real* __restr
   for (int j = 1; j <= D; ++j) ke += ub[j] * ub[j];
   const Real pb = gm1 * (ub[D + 1] - Real(0.5) * ke / ub[0]);
   if (!(ub[0] > Real(0) && pb > Real(0))) {
-    atomicExch(status, -4);
+    atomicExch(status, kStatusNonFinite);
     return;
   }
-  const Real eps_r = eps * ub[0], eps_p = eps * pb;
-  // check point k: volume point k < Q, else face point (k - Q) of face f
+  const Real eps_r = eps * ub[0], eps_p = eps * pb, Ep = eps_p / gm1;
+  Real rmin = ub[0];
+  bool low = false;
+  auto look = [&](const Real (&x)[NV]) {
+    Real k2 = Real(0);
+#pragma unroll
+    for (int j = 1; j <= D; ++j) k2 += x[j] * x[j];
+    rmin = x[0] < rmin ? x[0] : rmin;
+    low = low || x[0] * (x[D + 1] - Ep) < Real(0.5) * k2;
+  };
+#pragma unroll
+  for (int a = 0; a < D; ++a)
+#pragma unroll(C::REGS ? NFP : 3)
+    for (int fp = 0; fp < NFP; ++fp) {
+      Real lo[NV], up[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) lo[v] = up[v] = Real(0);
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        Real x[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          x[v] = X(v, face_point_index<D, N>(a, fp, k));
+          lo[v] += T.lm[k] * x[v];
+          up[v] += T.lp[k] * x[v];
+        }
+        if (a == 0) look(x);
+      }
+      look(lo);
+      look(up);
+    }
+  if (rmin >= eps_r && !low) return;
+
+  // limited: theta from every check point k (volume point k < Q, else face
+  // point (k - Q) of face f)
   auto point = [&](int k, Real (&x)[NV]) {
     if (k < Q) {
 #pragma unroll
@@ -1880,14 +1941,9 @@ __global__ void k_limit(int nL, int n, Real* __restrict__ U, const Real* __restr
     }
   };
   constexpr int NCHK = Q + 2 * D * NFP;
-  Real rmin = ub[0];
-  for (int k = 0; k < NCHK; ++k) {
-    Real x[NV];
-    point(k, x);
-    rmin = x[0] < rmin ? x[0] : rmin;
-  }
   const Real th1 = rmin >= eps_r ? Real(1) : fmin(Real(1), (ub[0] - eps_r) / (ub[0] - rmin));
   Real th2 = Real(1);
+#pragma unroll 1
   for (int k = 0; k < NCHK; ++k) {
     Real x[NV], du[NV];
     point(k, x);
@@ -1907,6 +1963,7 @@ __global__ void k_limit(int nL, int n, Real* __restrict__ U, const Real* __restr
   }
   const Real theta = th1 * th2;
   if (!(theta < Real(1))) return;
+#pragma unroll 1
   for (int q = 0; q < Q; ++q)
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -2124,7 +2181,7 @@ template <int D, int P, typename Real>
 struct LoadCfg {
   static constexpr int NV = D + 2, Q = ipow(P + 1, D);
   static constexpr int CT = NV * Q * 32 * (int)sizeof(Real) <= 46 * 1024 ? 32 : 16;
-  static constexpr int NT = CT * NV;
+  static constexpr int NT = (CT * NV + 31) / 32 * 32;  // whole warps: the reduction shuffles
 };
 template <int D, int P, typename Real>
 __global__ void __launch_bounds__(LoadCfg<D, P, Real>::NT) k_load_state(
@@ -2136,7 +2193,7 @@ __global__ void __launch_bounds__(LoadCfg<D, P, Real>::NT) k_load_state(
   const size_t g0 = (size_t)blockIdx.x * CT;
   const int lane = threadIdx.x % CT, v = threadIdx.x / CT;
   const size_t g = g0 + lane;
-  if (g < cells) {
+  if (g < cells && v < NV) {
     const size_t b = g / nc;
     const size_t off = (b * NV + v) * Q * nc + (g - b * nc);
     Real a[Q];

@@ -351,12 +351,13 @@ static cudaError_t indicator_p(const RtMisc& r, cudaStream_t s) {
 
 template <int D, int P, typename Real>
 static cudaError_t limit_p(const RtMisc& r, cudaStream_t s) {
-  const int nc = D == 3 ? r.n * r.n * r.n : r.n * r.n;
-  const size_t total = (size_t)r.nL * nc;
-  const int th = 128;
+  using C = LimitCfg<D, P, Real>;
+  int lnc = 0;
+  while ((1 << lnc) < (D == 3 ? r.n * r.n * r.n : r.n * r.n)) ++lnc;
+  const size_t total = (size_t)r.nL << lnc;
   if (total == 0) return cudaSuccess;
-  k_limit<D, P, Real><<<(unsigned)((total + th - 1) / th), th, 0, s>>>(
-      r.nL, r.n, (Real*)r.Uout, (const Real*)r.geo, r.affine, (Real)r.gamma, (Real)r.eps, r.status,
+  k_limit<D, P, Real><<<(unsigned)((total + C::NT - 1) / C::NT), C::NT, 0, s>>>(
+      r.nL, lnc, (Real*)r.Uout, (const Real*)r.geo, r.affine, (Real)r.gamma, (Real)r.eps, r.status,
       make_tab<P + 1, Real>(r.T));
   return cudaGetLastError();
 }
