@@ -235,6 +235,7 @@ struct StageArgs {
   const int* __restrict__ nbr;     // [b][f][4]
   const int* __restrict__ orient;  // [b][f] packed decoded orientation
   const int* __restrict__ qbits;   // [b] pos & 1 bits
+  const int* __restrict__ trd;     // [b][f][8] face-trace descriptors, see GuardArgs
   const double* __restrict__ dtp;
   unsigned long long* lam_bits;
   int* status;
@@ -368,6 +369,8 @@ struct GuardArgs {
   const int* __restrict__ fine_list;  // [nfine] leaf * 2D + face of every finer-neighbour face
   int nfine;
   const int* __restrict__ trd;        // [b][f][8] face-trace descriptors (kinds 0, 1, 3), see k_guard_trace
+  const int* __restrict__ tlist;      // [ntr] leaf * 2D + face of the faces to trace, null: every face
+  int ntr;
   // mortar mode (reading R15)
   const Real* __restrict__ geo;       // [b][g][cell] trilinear coefficients
   Real gamma;
@@ -1479,15 +1482,15 @@ __device__ __forceinline__ void guard_trace_block(const GuardArgs<D, P, Real>& A
   // launch keeps the thread count below 2^32)
   const int ln = 31 - __clz(n), lnt = (D - 1) * ln;
   if ((int)bid >= n_fine_blocks) {
-    const size_t total = (size_t)A.nL * 2 * D * nt * NV;
+    const size_t total = (size_t)A.ntr * nt * NV;
     const size_t wl = (size_t)(bid - n_fine_blocks) * NTH + threadIdx.x;
     if (wl >= total) return;
     const unsigned w = (unsigned)wl;
     const int t = (int)(w & (unsigned)(nt - 1));
     const unsigned r = w >> lnt;
     const int v = (int)(r % NV);
-    const int f = (int)((r / NV) % (2 * D));
-    const int b = (int)(r / (NV * 2 * D));
+    const int face = A.tlist ? __ldg(&A.tlist[r / NV]) : (int)(r / NV);
+    const int f = face % (2 * D), b = face / (2 * D);
     const int kind = A.kind[b * 2 * D + f];
     if (kind == 2) return;
     Real* out_trace = A.out + (((size_t)b * 2 * D + f) * NV + v) * NFP * nt + t;
@@ -2055,11 +2058,23 @@ __global__ void k_transfer(int nL, int n, const Real* __restrict__ old, Real* __
 
 // ============================================================ conversions
 // Modal <-> nodal along one axis of a cell's M values, in place, one line at
-// a time.  P_k(-x) = (-1)^k P_k(x) and the Gauss points are symmetric, so a
-// point pair (q, N-1-q) shares its even and its odd part, and P_0 = 1: 4
-// multiply-adds per line of 3 to nodes and 7 back instead of 9 (2 and 4 of
-// 4 at N = 2, 10 and 12 of 16 at N = 4).  In FP64 the transforms are bound
-// by the multiply-add rate (2 per clock and SM), so that is their time.
+// a time.  FP32 (bound by memory) takes the plain sums in mode order.  FP64
+// is bound by its multiply-adds (2 per clock and SM): P_k(-x) = (-1)^k P_k(x)
+// and the Gauss points are symmetric, so a point pair (q, N-1-q) shares its
+// even and its odd part, and P_0 = 1: 4 multiply-adds per line of 3 to nodes
+// and 7 back instead of 9 (2 and 4 of 4 at N = 2, 10 and 12 of 16 at N = 4).
+template <int N, typename Real>
+__device__ __forceinline__ void line_plain(const Real (&A)[N][N], Real (&u)[N]) {
+  Real r[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    r[i] = Real(0);
+#pragma unroll
+    for (int k = 0; k < N; ++k) r[i] += A[i][k] * u[k];
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) u[i] = r[i];
+}
 template <int N, typename Real>
 __device__ __forceinline__ void line_to_nodal(const Real (&V)[N][N], Real (&u)[N]) {
   Real r[N];
@@ -2124,7 +2139,8 @@ __device__ __forceinline__ void transform_cell(const Tab<N, Real>& T, Real (&a)[
       Real l[N];
 #pragma unroll
       for (int k = 0; k < N; ++k) l[k] = a[o + k * S];
-      if constexpr (TO_NODAL) line_to_nodal<N, Real>(T.V, l);
+      if constexpr (sizeof(Real) == 4) line_plain<N, Real>(TO_NODAL ? T.V : T.Vi, l);
+      else if constexpr (TO_NODAL) line_to_nodal<N, Real>(T.V, l);
       else line_to_modal<N, Real>(T.Vi, l);
 #pragma unroll
       for (int k = 0; k < N; ++k) a[o + k * S] = l[k];

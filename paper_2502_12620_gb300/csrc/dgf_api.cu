@@ -203,8 +203,9 @@ struct dgf_forest {
   Buf Uhi, Ulo;  // compensated form: u^n as the FP32 pair hi + lo, split once per step
   cudaGraphExec_t graph_alt = nullptr;  // compensated form: graph of the other u^n buffer
   Buf U[3], geo, geo64, hcell, gtr, gmod, cop, ctr, kind, nbr, orient, qbits, copoff, part, scal, tot,
-      dtout, nodal, fine, affine, ameta, trd;
+      dtout, nodal, fine, affine, ameta, trd, tlist;
   int nfine = 0;
+  int ntr = 0;  // faces of tlist: coarser neighbours and prescribed states
   // mortar treatment of level jumps (reading R15)
   bool mortar = false;
   Buf fluxmask, mfine, mcoarse, mw, msrc;
@@ -373,9 +374,9 @@ bool grid_env(bool dflt) {
 }
 
 // the cell-pair FP32 stage kernel covers 3D forests of 8^3-cell blocks at
-// p = 1, 2 in plain FP32
+// p = 1..3 in plain FP32
 bool pair_applies(const dgf_forest* f) {
-  return f->d == 3 && f->n == 8 && (f->p == 1 || f->p == 2) && f->precision == DGF_FP32 && !f->comp;
+  return f->d == 3 && f->n == 8 && f->p >= 1 && f->p <= 3 && f->precision == DGF_FP32 && !f->comp;
 }
 
 // Build every leaf-dependent device array: integer tables, FP64 geometry,
@@ -482,6 +483,13 @@ dgf_status build_device(dgf_forest* f) {
         e[7] = ipw(Nq, b2) * nc * 2 + s2;
       }
   }
+
+  // faces whose traces the guard pass computes for every stage kernel
+  std::vector<int> tlist;
+  for (int64_t i = 0; i < L * nf; ++i)
+    if (kind[i] == kCoarser || kind[i] == 4) tlist.push_back((int)i);
+  f->ntr = (int)tlist.size();
+  if (tlist.empty()) tlist.push_back(0);  // a non-null list of no faces
 
   // geometry: per-cell trilinear coefficients (c >= 1) and sizes h; the
   // leaves are independent, so host threads take them in any order
@@ -810,7 +818,8 @@ dgf_status build_device(dgf_forest* f) {
   }
   if ((st = upload(f, f->kind, kind)) || (st = upload(f, f->nbr, nbr)) || (st = upload(f, f->orient, orient)) ||
       (st = upload(f, f->qbits, qbits)) || (st = upload(f, f->copoff, copoff)) || (st = upload(f, f->geo64, geo64)) ||
-      (st = upload(f, f->fine, fine_list)) || (st = upload(f, f->trd, trd)))
+      (st = upload(f, f->fine, fine_list)) || (st = upload(f, f->trd, trd)) ||
+      (st = upload(f, f->tlist, tlist)))
     return st;
   if ((st = upload(f, f->affine, affine)) || (st = upload(f, f->hcell64, hcell))) return st;
   f->all_affine = std::all_of(affine.begin(), affine.end(), [](unsigned char a) { return a != 0; });
@@ -918,6 +927,7 @@ RtStage stage_args(dgf_forest* f, int src, int dst, double ca, double cb, int mo
   r.nbr = (const int*)f->nbr.ptr;
   r.orient = (const int*)f->orient.ptr;
   r.qbits = (const int*)f->qbits.ptr;
+  r.trd = (const int*)f->trd.ptr;
   r.U = f->U[src].ptr;
   r.Un = f->U[0].ptr;
   r.Uout = f->U[dst].ptr;
@@ -945,7 +955,13 @@ RtStage stage_args(dgf_forest* f, int src, int dst, double ca, double cb, int mo
   return r;
 }
 
-RtGuard guard_args(dgf_forest* f, int src, void* out, int mode) {
+// Does the stage kernel evaluate the traces of same-level and outflow faces
+// itself?  The cell-pair kernel does; then the guard pass of a time step only
+// covers level jumps and prescribed states (tlist).
+bool stage_traces(const dgf_forest* f, int kernel) { return pair_applies(f) && kernel != 1; }
+
+// kernel: the stage kernel that follows (its traces are left out of the pass)
+RtGuard guard_args(dgf_forest* f, int src, void* out, int mode, int kernel) {
   RtGuard r{};
   r.p = f->p;
   r.nL = (int)f->nL;
@@ -963,6 +979,10 @@ RtGuard guard_args(dgf_forest* f, int src, void* out, int mode) {
   r.fine_list = (const int*)f->fine.ptr;
   r.nfine = f->nfine;
   r.trd = (const int*)f->trd.ptr;
+  if (mode == 1 && stage_traces(f, kernel)) {
+    r.tlist = (const int*)f->tlist.ptr;
+    r.ntr = f->ntr;
+  }
   r.geo = f->geo.ptr;
   r.gamma = f->gamma;
   r.bstate = f->bstate.ptr;
@@ -1138,7 +1158,7 @@ dgf_status autotune(dgf_forest* f) {
     }
   }
   dgf_status st = cuda_check(split_state(f), "split");
-  if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gtr.ptr, 1)), "guard");
+  if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gtr.ptr, 1, 1)), "guard");  // every face, for every candidate
   if (st) return st;
   std::vector<int> kernels;
   const char* ks = getenv("DGF_STAGE_KERNEL");
@@ -1209,7 +1229,8 @@ dgf_status autotune(dgf_forest* f) {
 dgf_status enqueue_step(dgf_forest* f) {
   DevScalars* s = (DevScalars*)f->scal.ptr;
   // kernels one call launches: the guard call adds the mortar passes
-  const int guard_kernels = 1 + (f->mortar && f->nmf > 0) + (f->mortar && f->nmc > 0);
+  const bool traced = stage_traces(f, f->kernel) && f->ntr == 0 && (f->mortar || f->nfine == 0);
+  const int guard_kernels = (traced ? 0 : 1) + (f->mortar && f->nmf > 0) + (f->mortar && f->nmc > 0);
   auto rec = [&](int cls, auto&& launch, int kernels = 1) -> dgf_status {
     cudaEvent_t a = nullptr, b = nullptr;
     if (f->timing) {
@@ -1237,7 +1258,7 @@ dgf_status enqueue_step(dgf_forest* f) {
   const int src[3] = {0, 1, 2}, dst[3] = {1, 2, 0};
   const double ca[3] = {0.0, 0.75, 1.0 / 3.0}, cb[3] = {1.0, 0.25, 2.0 / 3.0};
   for (int k = 0; k < 3; ++k) {
-    if ((st = rec(1, [&]() { return do_guard(f, guard_args(f, src[k], f->gtr.ptr, 1)); }, guard_kernels)))
+    if ((st = rec(1, [&]() { return do_guard(f, guard_args(f, src[k], f->gtr.ptr, 1, f->kernel)); }, guard_kernels)))
       return st;
     if ((st = rec(2, [&]() { return do_stage(f, stage_args(f, src[k], dst[k], ca[k], cb[k], 0, k == 2)); })))
       return st;
@@ -1388,7 +1409,7 @@ dgf_status dgf_forest_destroy(dgf_forest* f) {
                                &f->gmod, &f->cop, &f->ctr, &f->kind, &f->nbr, &f->orient, &f->qbits, &f->copoff,
                                &f->part, &f->scal, &f->tot, &f->dtout, &f->nodal, &f->fine, &f->affine, &f->ameta,
                                &f->U64[0], &f->U64[1], &f->hcell64, &f->gmod64, &f->Uhi, &f->Ulo, &f->fluxmask,
-                               &f->mfine, &f->mcoarse, &f->mw, &f->msrc, &f->ind, &f->bstate, &f->trd};
+                               &f->mfine, &f->mcoarse, &f->mw, &f->msrc, &f->ind, &f->bstate, &f->trd, &f->tlist};
     for (auto* b : bufs) dev_free(f, *b);
     if (f->own_stream && f->stream) cudaStreamDestroy(f->stream);
   }
@@ -1649,7 +1670,7 @@ dgf_status dgf_fill_guardcells(dgf_forest* f, void* guard, int is_device) {
   const size_t count = (size_t)f->nL * 2 * f->d * f->nv * f->M * f->nt;
   if (!ensure(f, f->gmod, count * f->esize)) return fail(DGF_ENOMEM, "guard allocation failed");
   dgf_status st = cuda_check(split_state(f), "split");
-  if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gmod.ptr, 0)), "guard");
+  if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gmod.ptr, 0, f->kernel)), "guard");
   if (st) return st;
   const bool dbl = f->precision == DGF_FP64;
   if ((st = cuda_check(do_convert(f, f->gmod.ptr, f->gmod.ptr, (size_t)f->nL * 2 * f->d, f->nt, 0, dbl), "to modal"))) return st;
@@ -1668,7 +1689,7 @@ dgf_status dgf_dg_residual(dgf_forest* f, void* dst, int is_device) {
   if (!f->have_state) return fail(DGF_ESTATE, "no state set");
   DeviceGuard dg(f->device);
   dgf_status st = cuda_check(split_state(f), "split");
-  if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gtr.ptr, 1)), "guard");
+  if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gtr.ptr, 1, f->kernel)), "guard");
   if (st) return st;
   if ((st = cuda_check(do_stage(f, stage_args(f, 0, 1, 0.0, 1.0, 1, 0)), "stage"))) return st;
   const bool dbl = f->precision == DGF_FP64;
@@ -2159,7 +2180,7 @@ extern "C" dgf_status dgf_dg_residual_noalloc(dgf_forest* f, const void* U_nodal
   void* scratch = nullptr;
   dgf_status st = noalloc_scratch(f->device, &scratch);
   if (st) return st;
-  RtGuard g = guard_args(f, 0, scratch, 1);
+  RtGuard g = guard_args(f, 0, scratch, 1, f->kernel);
   g.U = U_nodal;
   if ((st = cuda_check(do_guard(f, g), "guard"))) return st;
   RtStage s = stage_args(f, 0, 1, 0.0, 1.0, 1, 0);
@@ -2359,7 +2380,7 @@ dgf_status dgf_batch_set(dgf_batch* b, dgf_forest* const* forests, const double*
     for (int k = 0; k < 3; ++k) {
       rs[k].push_back(stage_args(f, src[k], dst[k], ca[k], cb[k], 0, k == 2));
       rs[k].back().zchunk = b->zchunk;
-      rg[k].push_back(guard_args(f, src[k], f->gtr.ptr, 1));
+      rg[k].push_back(guard_args(f, src[k], f->gtr.ptr, 1, b->kernel));
     }
     const int it = stage_items<3, float>(rs[0].back());
     if (it < 0) return fail(DGF_EUNSUPPORTED, "batch member tiling");

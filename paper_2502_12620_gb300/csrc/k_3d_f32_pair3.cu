@@ -1,0 +1,8 @@
+// The cell-pair FP32 stage kernel for 3D blocks of 8^3 cells at p = 3.
+#include "stage_pair.cuh"
+
+namespace dgf {
+template cudaError_t stage_pair_launch<3>(const StageArgs<3, 3, float>&, int, bool, bool, cudaStream_t, int);
+template int stage_pair_blocks_per_sm<3>(int);
+template cudaError_t stage_pair_launch_batch<3>(const StageArgs<3, 3, float>&, int, bool, cudaStream_t);
+}  // namespace dgf

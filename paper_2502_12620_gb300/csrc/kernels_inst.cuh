@@ -78,10 +78,10 @@ bool stage_mortar_prepare(size_t smem);
   DGF_INSTANTIATE_MORTAR_P(DIM, 3, REAL)
 
 // The cell-pair FP32 stage kernel (stage_pair.cuh) serves 3D forests of 8^3-cell
-// blocks at p = 1, 2 in plain FP32 (RtStage::kernel 0); k_stage serves the rest.
+// blocks at p = 1..3 in plain FP32 (RtStage::kernel 0); k_stage serves the rest.
 template <int D, int P, int NS, typename Real>
 constexpr bool pair_shape() {
-  return D == 3 && NS == 8 && (P == 1 || P == 2) && std::is_same<Real, float>::value;
+  return D == 3 && NS == 8 && P >= 1 && P <= 3 && std::is_same<Real, float>::value;
 }
 // launch and occupancy of the cell-pair kernel (k_3d_f32_pair<P>.cu); v
 // selects its CTA shape (p = 1: 0 four CTAs per SM, 1 five)
@@ -151,7 +151,7 @@ static cudaError_t stage_ns(const StageArgs<D, P, Real>& a, int slots, int comp,
   if constexpr (pair_shape<D, P, NS, Real>()) {
     if (!comp && (kernel == 0 || kernel == 2)) {
       const int g = a.nL * a.nchunks < slots ? a.nL * a.nchunks : slots;
-      if constexpr (P == 1 || P == 2)
+      if constexpr (P >= 1 && P <= 3)
         return stage_pair_launch<P>(a, g, a.fluxmask != nullptr, all_affine != 0, s, kernel == 2 ? 1 : 0);
     }
   }
@@ -186,6 +186,7 @@ static StageArgs<D, P, Real> make_stage_args(const RtStage& r) {
   a.nbr = r.nbr;
   a.orient = r.orient;
   a.qbits = r.qbits;
+  a.trd = r.trd;
   a.dtp = r.dtp;
   a.lam_bits = r.lam_bits;
   a.status = r.status;
@@ -241,6 +242,8 @@ static GuardArgs<D, P, Real> make_guard_args(const RtGuard& r) {
   a.fine_list = r.fine_list;
   a.nfine = r.nfine;
   a.trd = r.trd;
+  a.tlist = r.tlist;
+  a.ntr = r.tlist ? r.ntr : r.nL * 2 * D;
   a.geo = (const Real*)r.geo;
   a.gamma = (Real)r.gamma;
   a.mfine = r.mfine;
@@ -262,10 +265,11 @@ static cudaError_t guard_p(const RtGuard& r, cudaStream_t s) {
     // time-step path: traces of every face kind in one launch (finer faces
     // by the combine blocks unless the mortar passes replace them)
     constexpr int NTH = 32 << D;
-    const size_t items = (size_t)r.nL * 2 * D * (D + 2) * nt;
+    const size_t items = (size_t)a.ntr * (D + 2) * nt;
     if (items >= ((size_t)1 << 32)) return cudaErrorInvalidConfiguration;  // the kernel indexes in 32 bits
     const size_t ntb = (items + NTH - 1) / NTH;
     const int nfb = r.nfine * nt;
+    if (ntb + nfb == 0) return cudaSuccess;  // every face is traced by the stage kernel
     const bool comp = std::is_same<Real, float>::value && r.comp;
     if constexpr (std::is_same<Real, float>::value) {
       if (comp) k_guard_trace<D, P, Real, true><<<(unsigned)(ntb + nfb), NTH, 0, s>>>(a, nfb);
@@ -430,7 +434,7 @@ template <int D, int P, typename Real>
 static long long guard_blocks_p(const RtGuard& r, int* nfb) {
   constexpr int NTH = 32 << D;
   const int nt = D == 3 ? r.n * r.n : r.n;
-  const size_t items = (size_t)r.nL * 2 * D * (D + 2) * nt;
+  const size_t items = (size_t)(r.tlist ? r.ntr : r.nL * 2 * D) * (D + 2) * nt;
   *nfb = r.nfine * nt;
   return (long long)((items + NTH - 1) / NTH) + *nfb;
 }
@@ -438,7 +442,7 @@ static long long guard_blocks_p(const RtGuard& r, int* nfb) {
 template <int D, int P, typename Real>
 static int stage_batch_blocks_per_sm_p(int kernel, int all_affine) {
   if constexpr (D == 3 && std::is_same<Real, float>::value) {
-    if constexpr (P == 1 || P == 2) {
+    if constexpr (P >= 1 && P <= 3) {
       if (kernel == 0) return stage_pair_blocks_per_sm<P>(0);
     }
     constexpr int YS = stage_rows<D, P, Real>(8);
@@ -464,7 +468,7 @@ static cudaError_t launch_stage_batch_p(const RtStage& common, const void* membe
     a.members = reinterpret_cast<const StageArgs<D, P, Real>*>(members);
     a.istart = istart;
     a.nmem = nmem;
-    if constexpr (P == 1 || P == 2) {
+    if constexpr (P >= 1 && P <= 3) {
       if (common.kernel == 0) return stage_pair_launch_batch<P>(a, grid, common.all_affine != 0, s);
     }
     constexpr int YS = stage_rows<D, P, Real>(8);
@@ -479,7 +483,8 @@ template <int D, int P, typename Real>
 static cudaError_t launch_guard_batch_p(const void* members, const int* bstart, const int* nfb, int nmem,
                                         long long blocks, cudaStream_t s) {
   if constexpr (D == 3 && std::is_same<Real, float>::value) {
-    if (blocks <= 0 || blocks >= (1ll << 31)) return cudaErrorInvalidConfiguration;
+    if (blocks < 0 || blocks >= (1ll << 31)) return cudaErrorInvalidConfiguration;
+    if (blocks == 0) return cudaSuccess;  // every face is traced by the stage kernel
     k_guard_trace_batch<D, P, Real><<<(unsigned)blocks, 32 << D, 0, s>>>(
         reinterpret_cast<const GuardArgs<D, P, Real>*>(members), bstart, nfb, nmem);
     return cudaGetLastError();

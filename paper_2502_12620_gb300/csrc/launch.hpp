@@ -29,6 +29,7 @@ struct RtStage {
   const int* nbr;
   const int* orient;
   const int* qbits;
+  const int* trd;  // [leaf][face][8] face-trace descriptors
   const double* dtp;
   unsigned long long* lam_bits;
   int* status;
@@ -63,6 +64,8 @@ struct RtGuard {
   const int* fine_list;
   int nfine;
   const int* trd;  // [leaf][face][8] face-trace descriptors (kinds 0, 1, 3)
+  const int* tlist;  // mode 1: [ntr] faces to trace (leaf * 2D + face); null: every face
+  int ntr;
   // mortar mode: fine-side and coarse-side faces, coarse-side weights/sources
   const void* geo;
   double gamma;
