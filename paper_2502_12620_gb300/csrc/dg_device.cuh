@@ -147,19 +147,20 @@ __device__ __forceinline__ Real jacobian_det(const Real (&t)[D][D]) {
 
 // ------------------------------------------------------------------ Euler
 // Flux along an (unnormalised) vector a: F . a  (Eq. (2), Eq. (23)).
+// ri = 1 / rho.
 template <int D, typename Real>
-__device__ __forceinline__ void flux_along(const Real (&u)[D + 2], const Real (&a)[D], Real gm1,
+__device__ __forceinline__ void flux_along(const Real (&u)[D + 2], const Real (&a)[D], Real ri, Real gm1,
                                            Real (&F)[D + 2]) {
-  const Real ri = Real(1) / u[0];
   Real vn = Real(0), ke = Real(0);
 #pragma unroll
   for (int j = 0; j < D; ++j) {
     vn += u[1 + j] * a[j];
     ke += u[1 + j] * u[1 + j];
   }
+  if constexpr (sizeof(Real) == 8) F[0] = vn;
   vn *= ri;
+  if constexpr (sizeof(Real) == 4) F[0] = u[0] * vn;
   const Real p = gm1 * (u[D + 1] - Real(0.5) * ke * ri);
-  F[0] = u[0] * vn;
 #pragma unroll
   for (int j = 0; j < D; ++j) F[1 + j] = u[1 + j] * vn + p * a[j];
   F[D + 1] = (u[D + 1] + p) * vn;
@@ -167,13 +168,15 @@ __device__ __forceinline__ void flux_along(const Real (&u)[D + 2], const Real (&
 
 // Lax-Friedrichs flux (Eq. (5), dissipative sign) times the face area
 // element: a = area vector pointing from L to R (|a| = dS / d(face ref)).
+// FP32 adds the two physical fluxes.  FP64 counts its multiply-adds (an SM has
+// 2 a clock; a reciprocal costs about ten, a root more): the sides share one
+// reciprocal, 1/(rho_L rho_R) times the other density, their fluxes are summed
+// term by term, and the sound speed takes the area into its root,
+// sqrt(gamma p / rho |a|^2).
 template <int D, typename Real>
 __device__ __forceinline__ void lf_flux(const Real (&uL)[D + 2], const Real (&uR)[D + 2],
                                         const Real (&a)[D], Real gamma, Real (&Fh)[D + 2]) {
   const Real gm1 = gamma - Real(1);
-  Real FL[D + 2], FR[D + 2];
-  flux_along<D, Real>(uL, a, gm1, FL);
-  flux_along<D, Real>(uR, a, gm1, FR);
   Real an2 = Real(0), vnL = Real(0), vnR = Real(0), keL = Real(0), keR = Real(0);
 #pragma unroll
   for (int j = 0; j < D; ++j) {
@@ -183,7 +186,27 @@ __device__ __forceinline__ void lf_flux(const Real (&uL)[D + 2], const Real (&uR
     keL += uL[1 + j] * uL[1 + j];
     keR += uR[1 + j] * uR[1 + j];
   }
+  if constexpr (sizeof(Real) == 8) {
+    const Real rr = Real(1) / (uL[0] * uR[0]), riL = rr * uR[0], riR = rr * uL[0];
+    const Real vL = vnL * riL, vR = vnR * riR;
+    const Real pL = gm1 * (uL[D + 1] - Real(0.5) * keL * riL);
+    const Real pR = gm1 * (uR[D + 1] - Real(0.5) * keR * riR);
+    const Real ga2 = gamma * an2;
+    const Real sL = fabs(vL) + sqrt(ga2 * pL * riL);
+    const Real sR = fabs(vR) + sqrt(ga2 * pR * riR);
+    const Real alpha = Real(0.5) * ((sL > sR || sL != sL) ? sL : sR);
+    const Real hL = Real(0.5) * vL, hR = Real(0.5) * vR, pp = Real(0.5) * (pL + pR);
+    Fh[0] = Real(0.5) * (vnL + vnR) + alpha * (uL[0] - uR[0]);
+#pragma unroll
+    for (int j = 1; j <= D; ++j)
+      Fh[j] = alpha * (uL[j] - uR[j]) + (uL[j] * hL + (uR[j] * hR + pp * a[j - 1]));
+    Fh[D + 1] = alpha * (uL[D + 1] - uR[D + 1]) + ((uL[D + 1] + pL) * hL + (uR[D + 1] + pR) * hR);
+    return;
+  }
   const Real riL = Real(1) / uL[0], riR = Real(1) / uR[0];
+  Real FL[D + 2], FR[D + 2];
+  flux_along<D, Real>(uL, a, riL, gm1, FL);
+  flux_along<D, Real>(uR, a, riR, gm1, FR);
   const Real pL = gm1 * (uL[D + 1] - Real(0.5) * keL * riL);
   const Real pR = gm1 * (uR[D + 1] - Real(0.5) * keR * riR);
   const Real an = sqrt(an2);
@@ -236,6 +259,11 @@ struct StageArgs {
   const int* __restrict__ orient;  // [b][f] packed decoded orientation
   const int* __restrict__ qbits;   // [b] pos & 1 bits
   const int* __restrict__ trd;     // [b][f][8] face-trace descriptors, see GuardArgs
+  // FP64 forests with curved blocks: J dxi/dx (rows, then 1/J) at the Gauss
+  // points [b][D*D+1][q][cell] and the rows at each cell's lower faces
+  // [b][D*D][face point][cell]; null: evaluated from geo
+  const Real* __restrict__ met;
+  const Real* __restrict__ fmet;
   const double* __restrict__ dtp;
   unsigned long long* lam_bits;
   int* status;
@@ -401,12 +429,12 @@ struct GuardArgs {
 template <int P, typename Real>
 struct StageCfg {
   static constexpr int NT = sizeof(Real) == 4 ? (P <= 1 ? DGF_STAGE_NT_F32_P1 : P <= 2 ? DGF_STAGE_NT_F32 : 512)
-                                              : (P <= 1 ? 512 : 256);
+                                              : 256;  // FP64: two warps a scheduler keep the pipe busy, no spills
   static constexpr int MINB = sizeof(Real) == 4 ? (P <= 1 ? DGF_STAGE_MINB_F32_P1 : P <= 2 ? 2 : 1) : 1;
 };
 
 // shared-memory footprint of the stage kernel (bytes): nodal layer, residual
-// layer, x- and y-face fluxes, carried z-face flux
+// layer, x- and y-face fluxes, carried z-face flux, reciprocal density (FP64)
 template <int D, int P, typename Real>
 __host__ __device__ constexpr size_t stage_smem(int n, int rows) {
   constexpr int N = P + 1, NV = D + 2, Q = ipow(N, D), NFP = ipow(N, D - 1);
@@ -415,7 +443,8 @@ __host__ __device__ constexpr size_t stage_smem(int n, int rows) {
   size_t rs = us;
   size_t fx = (size_t)NV * NFP * (n + 1) * rows, fy = (size_t)NV * NFP * (rows + 1) * n;
   size_t fz = D == 3 ? (size_t)NV * NFP * ncl : 0;
-  return (us + rs + fx + fy + fz) * sizeof(Real);
+  size_t ri = sizeof(Real) == 8 ? Q * ncl : 0;  // 1 / rho, FP64
+  return (us + rs + fx + fy + fz + ri) * sizeof(Real);
 }
 
 // rows of a layer one work item sweeps: the whole layer when its buffers fit
@@ -586,6 +615,7 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Real sx[N];
   __shared__ Real sam[D * D + 1];
+  constexpr bool SHRI = sizeof(Real) == 8;
   constexpr int RSZ = NV * Q * NCL;
   Real* us = reinterpret_cast<Real*>(smem_raw);
   Real* rs = us + NV * Q * NCL;
@@ -593,6 +623,7 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
   Real* fy = fx + NV * NFP * (n + 1) * YR;
   Real* fz = fy + NV * NFP * (YR + 1) * n;
   Real* tb = fx;   // halo traces reuse the x-face buffer when it is free
+  Real* rho1 = fz + (D == 3 ? NV * NFP * NCL : 0);  // [q][cell] 1 / rho (FP64)
   if (tid < N) sx[tid] = T.x[tid];
 
   Real lam_min = Real(3.0e38);
@@ -639,6 +670,12 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
     const int fmask = MORTAR ? M.fluxmask[b] : 0;  // faces whose flux is given (mortar mode)
     __syncthreads();  // previous item is done with the shared buffers
     if (aff && tid < D * D + 1) sam[tid] = M.ameta[(size_t)b * (D * D + 1) + tid];
+    // metric tables of a curved block
+    const bool tab = sizeof(Real) == 8 && !aff && M.met != nullptr;
+    const Real* __restrict__ Mb = tab ? M.met + (size_t)b * (D * D + 1) * Q * nc : nullptr;
+    const Real* __restrict__ Fb = tab ? M.fmet + (size_t)b * D * D * NFP * nc : nullptr;
+#define MET(g, q, c) __ldg(&Mb[((g) * Q + (q)) * nc + (c)])
+#define FMET(a, j, fp, c) __ldg(&Fb[(((a) * D + (j)) * NFP + (fp)) * nc + (c)])
 
     for (int k = k0; k < k1; ++k) {
       const int cbase = (D == 3 ? k * LAY : 0) + j0 * n;  // first cell of the slab
@@ -671,6 +708,14 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
           Real x[VEC];
           Sb.template vec<VEC>((size_t)r * nc + cbase + cv, x);
           vstore<VEC>(reinterpret_cast<V4*>(us + r * NCL + cv), x);
+          if constexpr (SHRI) {
+            if (r < Q) {  // the density rows
+              Real y[VEC];
+#pragma unroll
+              for (int e = 0; e < VEC; ++e) y[e] = Real(1) / x[e];
+              vstore<VEC>(reinterpret_cast<V4*>(rho1 + r * NCL + cv), y);
+            }
+          }
         }
       }
       if constexpr (D == 3) {
@@ -722,6 +767,9 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
             if (aff) {
 #pragma unroll
               for (int j = 0; j < 3; ++j) Ja[j] = sam[6 + j];
+            } else if (tab) {
+#pragma unroll
+              for (int j = 0; j < 3; ++j) Ja[j] = FMET(2, j, fp, cbase + c);
             } else if (k0 == 0) {
               const Real xi[3] = {sx[fp % N], sx[fp / N], Real(-1)};
               point_row<3, Real>(Gk + c, nc, xi, 2, Ja);
@@ -780,6 +828,9 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
           if (aff) {
 #pragma unroll
             for (int jj = 0; jj < D; ++jj) Ja[jj] = sam[jj];
+          } else if (tab && fi < n) {
+#pragma unroll
+            for (int jj = 0; jj < D; ++jj) Ja[jj] = FMET(0, jj, fp, cbase + cr);
           } else {
             Real xi[D];
             xi[0] = fi == n ? Real(1) : Real(-1);
@@ -839,6 +890,9 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
           if (aff) {
 #pragma unroll
             for (int jj = 0; jj < D; ++jj) Ja[jj] = sam[D + jj];
+          } else if (tab && !top) {
+#pragma unroll
+            for (int jj = 0; jj < D; ++jj) Ja[jj] = FMET(1, jj, fp, cbase + cr);
           } else {
             Real xi[D];
             xi[0] = sx[qx];
@@ -861,7 +915,7 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
         xi[1] = sx[fp % N];
         if constexpr (D == 3) xi[2] = sx[fp / N];
         LineGeo<D, 0, Real> lg;
-        if (!aff) lg.init(Gk + c, nc, xi);
+        if (!aff && !tab) lg.init(Gk + c, nc, xi);
         Real F[N][NV];
 #pragma unroll
         for (int qx = 0; qx < N; ++qx) {
@@ -871,10 +925,13 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
           if (aff) {
 #pragma unroll
             for (int jj = 0; jj < D; ++jj) Ja[jj] = sam[jj];
+          } else if (tab) {
+#pragma unroll
+            for (int jj = 0; jj < D; ++jj) Ja[jj] = MET(jj, qx + N * fp, cbase + c);
           } else {
             lg.at(T.x[qx], Ja);
           }
-          flux_along<D, Real>(u, Ja, gm1, Fq);
+          flux_along<D, Real>(u, Ja, SHRI ? rho1[(qx + N * fp) * NCL + c] : Real(1) / u[0], gm1, Fq);
 #pragma unroll
           for (int v = 0; v < NV; ++v) F[qx][v] = Fq[v];
         }
@@ -909,7 +966,7 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
           xi[1] = Real(0);
           if constexpr (D == 3) xi[2] = sx[qz];
           LineGeo<D, 1, Real> lg;
-          if (!aff) lg.init(Gk + c, nc, xi);
+          if (!aff && !tab) lg.init(Gk + c, nc, xi);
           Real F[N][NV];
           Real iJ[N];
 #pragma unroll
@@ -922,11 +979,15 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
 #pragma unroll
               for (int jj = 0; jj < D; ++jj) Ja[jj] = sam[D + jj];
               iJ[qy] = sam[D * D];
+            } else if (tab) {
+#pragma unroll
+              for (int jj = 0; jj < D; ++jj) Ja[jj] = MET(D + jj, q, cbase + c);
+              if constexpr (D == 2) iJ[qy] = MET(D * D, q, cbase + c);
             } else {
               lg.at(T.x[qy], Ja);
               if constexpr (D == 2) iJ[qy] = Real(1) / lg.jac(Ja);
             }
-            flux_along<D, Real>(u, Ja, gm1, Fq);
+            flux_along<D, Real>(u, Ja, SHRI ? rho1[q * NCL + c] : Real(1) / u[0], gm1, Fq);
 #pragma unroll
             for (int v = 0; v < NV; ++v) F[qy][v] = Fq[v];
           }
@@ -976,7 +1037,7 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
           const int qx = fp % N, qy = fp / N;
           const Real xi[3] = {sx[qx], sx[qy], Real(0)};
           LineGeo<3, 2, Real> lg;
-          if (!aff) lg.init(Gk + c, nc, xi);
+          if (!aff && !tab) lg.init(Gk + c, nc, xi);
           Real F[N][NV];
           Real iJ[N];
 #pragma unroll
@@ -988,11 +1049,15 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
 #pragma unroll
               for (int jj = 0; jj < 3; ++jj) Ja[jj] = sam[6 + jj];
               iJ[qz] = sam[9];
+            } else if (tab) {
+#pragma unroll
+              for (int jj = 0; jj < 3; ++jj) Ja[jj] = MET(6 + jj, fp + NFP * qz, cbase + c);
+              iJ[qz] = MET(9, fp + NFP * qz, cbase + c);
             } else {
               lg.at(T.x[qz], Ja);
               iJ[qz] = Real(1) / lg.jac(Ja);
             }
-            flux_along<3, Real>(u, Ja, gm1, Fq);
+            flux_along<3, Real>(u, Ja, SHRI ? rho1[(fp + NFP * qz) * NCL + c] : Real(1) / u[0], gm1, Fq);
 #pragma unroll
             for (int v = 0; v < NV; ++v) F[qz][v] = Fq[v];
           }
@@ -1013,6 +1078,12 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
             if (aff) {
 #pragma unroll
               for (int jj = 0; jj < 3; ++jj) Ja[jj] = sam[6 + jj];
+            } else if (tab && k < n - 1) {  // the lower faces of the layer above
+#pragma unroll
+              for (int jj = 0; jj < 3; ++jj) Ja[jj] = FMET(2, jj, fp, cbase + LAY + c);
+            } else if (tab) {
+              const Real xt[3] = {sx[qx], sx[qy], Real(1)};
+              point_row<3, Real>(Gk + c, nc, xt, 2, Ja);
             } else {
               lg.at(Real(1), Ja);
             }
@@ -1132,6 +1203,8 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
 #undef TB
 #undef FZ
 #undef GTR
+#undef MET
+#undef FMET
 
   if (!BATCH && A.last) {
     // block min of h/lambda -> one atomic per CTA
@@ -2054,6 +2127,57 @@ __global__ void k_transfer(int nL, int n, const Real* __restrict__ old, Real* __
   }
 #pragma unroll
   for (int q = 0; q < Q; ++q) o[(size_t)q * nc] = acc[q];
+}
+
+// ============================================================ metric tables
+// J dxi/dx (rows) and 1/J at the Gauss points, and the rows at each cell's
+// lower faces, of every cell (StageArgs::met, fmet): once per build, so that
+// the FP64 stage kernel, bound by its 2 multiply-adds a clock and SM, does not
+// evaluate them three times a stage.  One thread per (leaf, cell).
+template <int D, int P, typename Real>
+__global__ void k_metric(int nL, int nc, const Real* __restrict__ geo, Real* __restrict__ met, Real* __restrict__ fmet,
+                         Tab<P + 1, Real> T) {
+  constexpr int N = P + 1, Q = ipow(N, D), NFP = ipow(N, D - 1), NG = ((1 << D) - 1) * D;
+  const size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (w >= (size_t)nL * nc) return;
+  const size_t b = w / nc;
+  const int c = (int)(w - b * nc);
+  const Real* X = geo + b * NG * nc + c;
+  Real* m = met + b * (D * D + 1) * Q * nc + c;
+  Real* f = fmet + b * D * D * NFP * nc + c;
+#pragma unroll 1
+  for (int q = 0; q < Q; ++q) {
+    Real xi[D], t[D][D], J = Real(0);
+    for (int a = 0, r = q; a < D; ++a, r /= N) xi[a] = T.x[r % N];
+    tangents<D, Real>(X, nc, xi, t);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      Real row[D];
+      contra_row<D, Real>(t, a, row);
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        m[(size_t)((a * D + j) * Q + q) * nc] = row[j];
+        if (a == 0) J += t[0][j] * row[j];
+      }
+    }
+    m[(size_t)(D * D * Q + q) * nc] = Real(1) / J;
+  }
+#pragma unroll 1
+  for (int i = 0; i < D * NFP; ++i) {
+    const int a = i / NFP, fp = i % NFP;
+    Real xi[D], row[D];
+    for (int ax = 0, r = fp; ax < D; ++ax) {
+      if (ax == a) {
+        xi[ax] = Real(-1);
+        continue;
+      }
+      xi[ax] = T.x[r % N];
+      r /= N;
+    }
+    point_row<D, Real>(X, nc, xi, a, row);
+#pragma unroll
+    for (int j = 0; j < D; ++j) f[(size_t)((a * D + j) * NFP + fp) * nc] = row[j];
+  }
 }
 
 // ============================================================ conversions

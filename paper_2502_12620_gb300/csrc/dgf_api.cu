@@ -203,7 +203,7 @@ struct dgf_forest {
   Buf Uhi, Ulo;  // compensated form: u^n as the FP32 pair hi + lo, split once per step
   cudaGraphExec_t graph_alt = nullptr;  // compensated form: graph of the other u^n buffer
   Buf U[3], geo, geo64, hcell, gtr, gmod, cop, ctr, kind, nbr, orient, qbits, copoff, part, scal, tot,
-      dtout, nodal, fine, affine, ameta, trd, tlist;
+      dtout, nodal, fine, affine, ameta, trd, tlist, met, fmet;
   int nfine = 0;
   int ntr = 0;  // faces of tlist: coarser neighbours and prescribed states
   // mortar treatment of level jumps (reading R15)
@@ -855,6 +855,32 @@ dgf_status build_device(dgf_forest* f) {
   if (!ensure(f, f->gtr, (size_t)L * nf * f->nv * f->NFP * nt * f->esize) ||
       !ensure(f, f->part, (size_t)L * nc * f->nv * sizeof(double)))
     return fail(DGF_ENOMEM, "scratch allocation failed");
+  // metric tables for FP64 forests with curved blocks, where memory allows
+  // (the stage kernel evaluates the metric itself without them)
+  if (f->precision == DGF_FP64 && !f->all_affine) {
+    const size_t cells = (size_t)L * nc;
+    if (ensure(f, f->met, cells * (d * d + 1) * M * sizeof(double)) &&
+        ensure(f, f->fmet, cells * d * d * f->NFP * sizeof(double))) {
+      RtMisc r{};
+      r.p = f->p;
+      r.nL = (int)L;
+      r.n = n;
+      r.T = f->tab;
+      r.geo = f->geo.ptr;
+      r.met = f->met.ptr;
+      r.fmet = f->fmet.ptr;
+      if ((st = cuda_check(d == 2 ? launch_metric<2, double>(r, f->stream) : launch_metric<3, double>(r, f->stream),
+                           "metric tables")))
+        return st;
+    } else {
+      cudaGetLastError();  // a refused cudaMalloc
+      dev_free(f, f->met);
+      dev_free(f, f->fmet);
+    }
+  } else {
+    dev_free(f, f->met);
+    dev_free(f, f->fmet);
+  }
   // resident stage CTAs, and the z-chunk length that balances the
   // persistent CTAs best (a chunk costs its layers plus ~0.3 layer of halo)
   {
@@ -928,6 +954,8 @@ RtStage stage_args(dgf_forest* f, int src, int dst, double ca, double cb, int mo
   r.orient = (const int*)f->orient.ptr;
   r.qbits = (const int*)f->qbits.ptr;
   r.trd = (const int*)f->trd.ptr;
+  r.met = f->met.ptr;
+  r.fmet = f->fmet.ptr;
   r.U = f->U[src].ptr;
   r.Un = f->U[0].ptr;
   r.Uout = f->U[dst].ptr;
@@ -1409,7 +1437,7 @@ dgf_status dgf_forest_destroy(dgf_forest* f) {
                                &f->gmod, &f->cop, &f->ctr, &f->kind, &f->nbr, &f->orient, &f->qbits, &f->copoff,
                                &f->part, &f->scal, &f->tot, &f->dtout, &f->nodal, &f->fine, &f->affine, &f->ameta,
                                &f->U64[0], &f->U64[1], &f->hcell64, &f->gmod64, &f->Uhi, &f->Ulo, &f->fluxmask,
-                               &f->mfine, &f->mcoarse, &f->mw, &f->msrc, &f->ind, &f->bstate, &f->trd, &f->tlist};
+                               &f->mfine, &f->mcoarse, &f->mw, &f->msrc, &f->ind, &f->bstate, &f->trd, &f->tlist, &f->met, &f->fmet};
     for (auto* b : bufs) dev_free(f, *b);
     if (f->own_stream && f->stream) cudaStreamDestroy(f->stream);
   }

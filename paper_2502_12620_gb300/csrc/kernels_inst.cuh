@@ -34,6 +34,25 @@ static Tab<N, Real> make_tab(const RtTables& r) {
   return t;
 }
 
+// Rows of a 2D block that one stage work item sweeps: the whole block, or a
+// quarter of it when that fills the SMs better.  An item costs its rows plus
+// about 1.5 rows (start-up and the slab's second edge faces), and the SM is
+// what items share (the FP64 pipe is the bound).  28 blocks of 8^2 cells,
+// p = 2, FP64, per stage: 43.5 us as 28 items, 24.7 us as 112 (with the FP64
+// sums of lf_flux).
+template <int NS>
+constexpr int slab_rows_2d() {
+  return NS >= 4 ? NS / 4 : NS;
+}
+template <int NS>
+static bool use_slabs_2d(int nL) {
+  constexpr int YS = slab_rows_2d<NS>(), SMS = 152;
+  if (YS == NS) return false;
+  const double whole = (double)((nL + SMS - 1) / SMS) * (NS + 1.5);
+  const double slabs = (double)(((long long)nL * (NS / YS) + SMS - 1) / SMS) * (YS + 1.5);
+  return slabs < whole;
+}
+
 // The mortar variants of the stage kernel (faces whose flux the mortar passes
 // give) live in their own translation units (k_<dim>_<prec>_mortar.cu).
 template <int D, int P, int NS, typename Real>
@@ -41,10 +60,31 @@ cudaError_t stage_mortar_launch(const StageArgs<D, P, Real>& a, int grid, size_t
 template <int D, int P, int NS, typename Real>
 bool stage_mortar_prepare(size_t smem);
 
+// 2D blocks in slabs, one CTA per slab
+template <int D, int P, int NS, typename Real, bool MORTAR>
+static cudaError_t stage_slab_launch(const StageArgs<D, P, Real>& a, int comp, cudaStream_t s) {
+  constexpr int YS = slab_rows_2d<NS>();
+  constexpr size_t smem = stage_smem<D, P, Real>(NS, YS);
+  static_assert(smem <= 48 * 1024, "no opt-in shared memory");
+  const int grid = a.nL * (NS / YS);
+  if constexpr (std::is_same<Real, float>::value) {
+    if (comp) {
+      k_stage<D, P, NS, Real, true, MORTAR, YS><<<grid, StageCfg<P, Real>::NT, smem, s>>>(a);
+      return cudaGetLastError();
+    }
+  }
+  if (comp) return cudaErrorInvalidValue;
+  k_stage<D, P, NS, Real, false, MORTAR, YS><<<grid, StageCfg<P, Real>::NT, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
 #define DGF_INSTANTIATE_MORTAR_NS(DIM, P, NS, REAL)                                                   \
   template <>                                                                                         \
   cudaError_t stage_mortar_launch<DIM, P, NS, REAL>(const StageArgs<DIM, P, REAL>& a, int grid,       \
                                                     size_t smem, int comp, cudaStream_t s) {          \
+    if constexpr (DIM == 2) {                                                                         \
+      if (use_slabs_2d<NS>(a.nL)) return stage_slab_launch<DIM, P, NS, REAL, true>(a, comp, s);       \
+    }                                                                                                 \
     if constexpr (std::is_same<REAL, float>::value) {                                                 \
       if (comp) {                                                                                     \
         k_stage<DIM, P, NS, REAL, true, true><<<grid, StageCfg<P, REAL>::NT, smem, s>>>(a);           \
@@ -156,6 +196,9 @@ static cudaError_t stage_ns(const StageArgs<D, P, Real>& a, int slots, int comp,
     }
   }
   if (a.fluxmask) return stage_mortar_launch<D, P, NS, Real>(a, grid, smem, comp, s);
+  if constexpr (D == 2) {
+    if (use_slabs_2d<NS>(a.nL)) return stage_slab_launch<D, P, NS, Real, false>(a, comp, s);
+  }
   if constexpr (std::is_same<Real, float>::value) {
     if (comp) {
       k_stage<D, P, NS, Real, true><<<grid, StageCfg<P, Real>::NT, smem, s>>>(a);
@@ -187,6 +230,8 @@ static StageArgs<D, P, Real> make_stage_args(const RtStage& r) {
   a.orient = r.orient;
   a.qbits = r.qbits;
   a.trd = r.trd;
+  a.met = (const Real*)r.met;
+  a.fmet = (const Real*)r.fmet;
   a.dtp = r.dtp;
   a.lam_bits = r.lam_bits;
   a.status = r.status;
@@ -385,6 +430,16 @@ static cudaError_t convert_p(size_t outer, int inner, const void* in, void* out,
   const int th = 128;
   k_convert<D, P, Real><<<(unsigned)((total + th - 1) / th), th, 0, s>>>(outer, inner, (const Real*)in, (Real*)out,
                                                                        to_nodal, make_tab<P + 1, Real>(T));
+  return cudaGetLastError();
+}
+
+template <int D, int P, typename Real>
+static cudaError_t metric_p(const RtMisc& r, cudaStream_t s) {
+  const int nc = D == 3 ? r.n * r.n * r.n : r.n * r.n;
+  const size_t total = (size_t)r.nL * nc;
+  if (total == 0) return cudaSuccess;
+  k_metric<D, P, Real><<<(unsigned)((total + 127) / 128), 128, 0, s>>>(
+      r.nL, nc, (const Real*)r.geo, (Real*)r.met, (Real*)r.fmet, make_tab<P + 1, Real>(r.T));
   return cudaGetLastError();
 }
 
@@ -594,6 +649,12 @@ static cudaError_t launch_guard_batch_p(const void* members, const int* bstart, 
     constexpr int D = DIM;                                                                  \
     using Real = REAL;                                                                      \
     DGF_DISPATCH_P(transfer_p, r, s)                                                        \
+  }                                                                                         \
+  template <>                                                                               \
+  cudaError_t launch_metric<DIM, REAL>(const RtMisc& r, cudaStream_t s) {                   \
+    constexpr int D = DIM;                                                                  \
+    using Real = REAL;                                                                      \
+    DGF_DISPATCH_P(metric_p, r, s)                                                          \
   }                                                                                         \
   template <>                                                                               \
   cudaError_t launch_load_state<DIM, REAL>(const RtMisc& r, cudaStream_t s) {               \

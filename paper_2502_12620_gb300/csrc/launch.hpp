@@ -30,6 +30,8 @@ struct RtStage {
   const int* orient;
   const int* qbits;
   const int* trd;  // [leaf][face][8] face-trace descriptors
+  const void* met;   // metric tables of an FP64 forest with curved blocks, or null
+  const void* fmet;
   const double* dtp;
   unsigned long long* lam_bits;
   int* status;
@@ -108,6 +110,8 @@ struct RtMisc {
   const void* geo;           // limiter: trilinear coefficients (compute precision)
   const unsigned char* affine;
   double eps;                // limiter bound, relative to the cell mean
+  void* met;                 // metric tables to fill
+  void* fmet;
   RtTables T;
 };
 
@@ -133,6 +137,9 @@ cudaError_t launch_transfer(const RtTransfer& r, cudaStream_t s);
 template <int D, typename Real>
 cudaError_t launch_convert(int p, size_t outer, int inner, const void* in, void* out, int to_nodal,
                            const RtTables& T, cudaStream_t s);
+// metric tables r.met, r.fmet from r.geo
+template <int D, typename Real>
+cudaError_t launch_metric(const RtMisc& r, cudaStream_t s);
 // modal state r.U -> nodal state r.Uout with its CFL minimum
 template <int D, typename Real>
 cudaError_t launch_load_state(const RtMisc& r, cudaStream_t s);
