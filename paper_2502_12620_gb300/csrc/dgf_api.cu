@@ -216,6 +216,9 @@ struct dgf_forest {
   // rebuild after a regrid reuses its pages
   hvec<double> h_geo64, h_hcell;
   hvec<float> h_geo32, h_hcell32;
+  // per leaf of the last build: affine block, and its constant 1/J
+  std::vector<unsigned char> h_affine;
+  std::vector<double> h_invj;
   // boundary faces: per root face 0 outflow, 1 prescribed state (bstate_h)
   std::vector<int32_t> bctag;
   std::vector<double> bstate_h;
@@ -522,46 +525,44 @@ dgf_status build_device(dgf_forest* f) {
       lo = hi;
     }
   }
-  parallel_for(L, [&](int64_t i) {
-    F.cell_coefficients(F.leaves[i], coef[i]);
-    for (int g = 0; g < NG; ++g)
-      for (int c = 0; c < nc; ++c) geo64[((size_t)i * NG + g) * nc + c] = coef[i][(size_t)(d + g) * nc + c];
-  });
-
-  // affine blocks: every cell a congruent parallelogram/parallelepiped ->
-  // constant J dxi/dx rows and 1/J per block
+  // one pass per leaf (a second or third one would start the host threads
+  // again and read the coefficients from memory again): coefficients; affine
+  // blocks, every cell a congruent parallelogram/parallelepiped -> constant
+  // J dxi/dx rows and 1/J per block; cell sizes h = (cell volume)^(1/d), the
+  // volume by the Gauss rule (an affine block's cells: J times the reference
+  // volume 2^d)
   std::vector<unsigned char> affine(L, 0);
   std::vector<double> ameta((size_t)L * (d * d + 1), 0.0);
-  parallel_for(L, [&](int64_t i) {
+  auto affine_meta = [&](int64_t i) -> bool {
     const std::vector<double>& C = coef[i];
     double scale = 0.0;
     for (int k = d; k < (1 << d) * d; ++k)
       for (int c = 0; c < nc; ++c) scale = std::max(scale, std::fabs(C[(size_t)k * nc + c]));
-    bool ok = scale > 0.0;
-    for (int cm = 1; cm < (1 << d) && ok; ++cm) {
+    if (!(scale > 0.0)) return false;
+    for (int cm = 1; cm < (1 << d); ++cm) {
       const bool linear = (cm & (cm - 1)) == 0;
-      for (int j = 0; j < d && ok; ++j) {
+      for (int j = 0; j < d; ++j) {
         const double* row = &C[((size_t)cm * d + j) * nc];
-        for (int c = 0; c < nc && ok; ++c) {
-          if (!linear && std::fabs(row[c]) > 1e-13 * scale) ok = false;
-          if (linear && std::fabs(row[c] - row[0]) > 1e-13 * scale) ok = false;
+        for (int c = 0; c < nc; ++c) {
+          if (!linear && std::fabs(row[c]) > 1e-13 * scale) return false;
+          if (linear && std::fabs(row[c] - row[0]) > 1e-13 * scale) return false;
         }
       }
     }
-    if (!ok) return;
     double cc[24], A[9], Ja[9], xi[3] = {0, 0, 0};
     for (int k = 0; k < (1 << d) * d; ++k) cc[k] = C[(size_t)k * nc];
     eval_map(d, cc, xi, nullptr, A);
     const double J = det_and_cofactor(d, A, Ja);
-    if (!(J > 0)) return;
-    affine[i] = 1;
+    if (!(J > 0)) return false;
     for (int k = 0; k < d * d; ++k) ameta[(size_t)i * (d * d + 1) + k] = Ja[k];
     ameta[(size_t)i * (d * d + 1) + d * d] = 1.0 / J;
-  });
-
-  // cell sizes h = (cell volume)^(1/d), the volume by the Gauss rule (an
-  // affine block's cells: J times the reference volume 2^d)
+    return true;
+  };
   parallel_for(L, [&](int64_t i) {
+    F.cell_coefficients(F.leaves[i], coef[i]);
+    for (int g = 0; g < NG; ++g)
+      for (int c = 0; c < nc; ++c) geo64[((size_t)i * NG + g) * nc + c] = coef[i][(size_t)(d + g) * nc + c];
+    affine[i] = affine_meta(i);
     if (affine[i]) {
       const double h = std::pow((double)(1 << d) / ameta[(size_t)i * (d * d + 1) + d * d], 1.0 / d);
       for (int c = 0; c < nc; ++c) hcell[(size_t)i * nc + c] = h;
@@ -586,6 +587,9 @@ dgf_status build_device(dgf_forest* f) {
       hcell[(size_t)i * nc + c] = std::pow(vol, 1.0 / d);
     }
   });
+  f->h_affine = affine;
+  f->h_invj.resize(L);
+  for (int64_t i = 0; i < L; ++i) f->h_invj[i] = ameta[(size_t)i * (d * d + 1) + d * d];
 
   // combine operators for every finer-neighbour guard cell (Eqs. (13)-(14),
   // J-weighted, integrals by each child's Gauss rule), rotated into my frame
@@ -1971,6 +1975,8 @@ static dgf_status regrid(dgf_forest* f, const std::vector<uint64_t>& old_leaves)
   dgf_forest::Buf& live = f->comp ? f->U64[f->cur] : f->U[0];
   old = live;
   live = dgf_forest::Buf();
+  const std::vector<unsigned char> old_affine = std::move(f->h_affine);
+  const std::vector<double> old_invj = std::move(f->h_invj);
   const bool was_tuned = f->tuned;
   const int tuned_z = f->zchunk, tuned_k = f->kernel;
   const bool tuned_g = f->grid_items;
@@ -2034,10 +2040,21 @@ static dgf_status regrid(dgf_forest* f, const std::vector<uint64_t>& old_leaves)
   }
   // combine operators (host, FP64): a parent cell whose children all have
   // the same constant Jacobian uses the shared reference operator (stored
-  // first); any other cell gets its own
+  // first); any other cell gets its own.  Children that are affine blocks of
+  // one Jacobian settle that for all cells of their parent, from what the
+  // last build kept (evaluating every child cell's map took 15 of the 30 ms
+  // of a refine and coarsen cycle on 120 to 253 affine blocks).
   const size_t opsz = (size_t)M * NW * M;
   std::vector<std::vector<double>> ccoef((size_t)combine_leaves.size() * NW);
+  std::vector<unsigned char> uniform(combine_leaves.size(), 0);
+  bool mixed = false;  // some parent needs its cells looked at
   for (size_t j = 0; j < combine_leaves.size(); ++j) {
+    const int* kd = &kids[(size_t)combine_leaves[j] * NW];
+    uniform[j] = old_affine.size() == old_leaves.size();
+    for (int c = 0; c < NW && uniform[j]; ++c)
+      if (!old_affine[kd[c]] || std::fabs(old_invj[kd[c]] - old_invj[kd[0]]) > 1e-12 * old_invj[kd[0]]) uniform[j] = 0;
+    if (uniform[j]) continue;
+    mixed = true;
     int64_t r;
     int lev, pos[3];
     Forest::unkey(f->host.leaves[combine_leaves[j]], &r, &lev, pos);
@@ -2066,7 +2083,8 @@ static dgf_status regrid(dgf_forest* f, const std::vector<uint64_t>& old_leaves)
   };
   // which cells need their own operator
   std::vector<unsigned char> own(ncomb, 0);
-  parallel_for(ncomb, [&](int64_t jc) {
+  parallel_for(mixed ? ncomb : 0, [&](int64_t jc) {
+    if (uniform[(size_t)(jc / nc)]) return;
     double cc[8][24];
     child_cells(jc, cc);
     double J0 = 0.0;
@@ -2101,7 +2119,7 @@ static dgf_status regrid(dgf_forest* f, const std::vector<uint64_t>& old_leaves)
     }
     if (!combine_op_cell(f, cp, &ops[0])) singular = true;
   }
-  parallel_for(ncomb, [&](int64_t jc) {
+  parallel_for(mixed ? ncomb : 0, [&](int64_t jc) {
     if (!own[jc]) return;
     double cc[8][24];
     const double* cp[8];
