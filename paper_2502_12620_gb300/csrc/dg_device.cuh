@@ -1692,7 +1692,8 @@ __device__ __forceinline__ void guard_trace_block(const GuardArgs<D, P, Real>& A
   for (int pr = lane; pr < NPAIR; pr += 32) {
     const int v = pr / NFP, fp = pr % NFP;
     Real acc0 = Real(0), acc1 = Real(0);
-#pragma unroll 4
+    // every load of the operator's column before the sums: one trip to L2
+#pragma unroll(Q <= 27 ? Q / 2 : 8)
     for (int q = 0; q + 1 < Q; q += 2) {
       acc0 += __ldg(&op[(size_t)q * NFP + fp]) * sv[e][v][q];
       acc1 += __ldg(&op[(size_t)(q + 1) * NFP + fp]) * sv[e][v][q + 1];

@@ -188,7 +188,10 @@ struct dgf_forest {
   size_t esize = 8;   // element size of the device compute buffers
   size_t sesize = 8;  // element size of the state at the C ABI
   bool comp = false;  // compensated form: u^n in FP64, stage increments in FP32
-  bool all_affine = false;  // every leaf an affine block (the stage kernel needs no per-cell geometry)
+  // every leaf an affine block (1: the stage kernel needs no per-cell geometry),
+  // and axis-aligned as well (2: nothing off the metric's diagonal, to the bit,
+  // so that leaving those terms out changes no bit)
+  int all_affine = 0;
   int cur = 0;        // compensated form: which U64 buffer holds u^n
   int d = 0, n = 0, p = 0, N = 0, nv = 0, M = 0, nc = 0, NG = 0, nt = 0, NFP = 0;
   int64_t nL = 0;
@@ -827,6 +830,13 @@ dgf_status build_device(dgf_forest* f) {
     return st;
   if ((st = upload(f, f->affine, affine)) || (st = upload(f, f->hcell64, hcell))) return st;
   f->all_affine = std::all_of(affine.begin(), affine.end(), [](unsigned char a) { return a != 0; });
+  if (f->all_affine) {
+    bool diag = true;
+    for (int64_t i = 0; i < L && diag; ++i)
+      for (int k = 0; k < d * d; ++k)
+        if (k % (d + 1) != 0 && ameta[(size_t)i * (d * d + 1) + k] != 0.0) diag = false;
+    if (diag) f->all_affine = 2;
+  }
   if (f->mortar && ((st = upload(f, f->fluxmask, fluxmask)) || (st = upload(f, f->mfine, mfine)) ||
                     (st = upload(f, f->mcoarse, mcoarse)) || (st = upload(f, f->msrc, msrc))))
     return st;
@@ -894,11 +904,11 @@ dgf_status build_device(dgf_forest* f) {
     for (int kk = 0; kk < 3; ++kk) {
       int occ = 0;
       if (d == 2)
-        occ = f->precision == DGF_FP64 ? stage_occupancy<2, double>(f->p, n, cp, kk)
-                                       : stage_occupancy<2, float>(f->p, n, cp, kk);
+        occ = f->precision == DGF_FP64 ? stage_occupancy<2, double>(f->p, n, cp, kk, f->all_affine)
+                                       : stage_occupancy<2, float>(f->p, n, cp, kk, f->all_affine);
       else
-        occ = f->precision == DGF_FP64 ? stage_occupancy<3, double>(f->p, n, cp, kk)
-                                       : stage_occupancy<3, float>(f->p, n, cp, kk);
+        occ = f->precision == DGF_FP64 ? stage_occupancy<3, double>(f->p, n, cp, kk, f->all_affine)
+                                       : stage_occupancy<3, float>(f->p, n, cp, kk, f->all_affine);
       f->slots_k[kk] = occ * sms;
     }
     if (!(pair_applies(f) && f->p == 1)) f->slots_k[2] = 0;
@@ -951,7 +961,7 @@ RtStage stage_args(dgf_forest* f, int src, int dst, double ca, double cb, int mo
   r.slots = f->grid_items ? INT_MAX : f->slots;  // the launch takes min(items, slots) CTAs
   r.kernel = f->kernel;
   r.affine = (const unsigned char*)f->affine.ptr;
-  r.all_affine = f->all_affine ? 1 : 0;
+  r.all_affine = f->all_affine;
   r.ameta = f->ameta.ptr;
   r.kind = (const int*)f->kind.ptr;
   r.nbr = (const int*)f->nbr.ptr;
@@ -2385,8 +2395,8 @@ dgf_status dgf_batch_set(dgf_batch* b, dgf_forest* const* forests, const double*
   b->kernel = pair_applies(f0) ? 0 : 1;
   if (const char* ks = getenv("DGF_STAGE_KERNEL"))
     if (strcmp(ks, "classic") == 0) b->kernel = 1;
-  b->all_affine = 1;
-  for (auto* f : b->mem) b->all_affine &= f->all_affine ? 1 : 0;
+  b->all_affine = 2;
+  for (auto* f : b->mem) b->all_affine = std::min(b->all_affine, f->all_affine);
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
   b->slots = stage_batch_blocks_per_sm<3, float>(b->p, b->kernel, b->all_affine) * sms;

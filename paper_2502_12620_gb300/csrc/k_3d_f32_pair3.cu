@@ -2,7 +2,7 @@
 #include "stage_pair.cuh"
 
 namespace dgf {
-template cudaError_t stage_pair_launch<3>(const StageArgs<3, 3, float>&, int, bool, bool, cudaStream_t, int);
-template int stage_pair_blocks_per_sm<3>(int);
-template cudaError_t stage_pair_launch_batch<3>(const StageArgs<3, 3, float>&, int, bool, cudaStream_t);
+template cudaError_t stage_pair_launch<3>(const StageArgs<3, 3, float>&, int, bool, int, cudaStream_t, int);
+template int stage_pair_blocks_per_sm<3>(int, int);
+template cudaError_t stage_pair_launch_batch<3>(const StageArgs<3, 3, float>&, int, int, cudaStream_t);
 }  // namespace dgf

@@ -124,24 +124,24 @@ constexpr bool pair_shape() {
   return D == 3 && NS == 8 && P >= 1 && P <= 3 && std::is_same<Real, float>::value;
 }
 // launch and occupancy of the cell-pair kernel (k_3d_f32_pair<P>.cu); v
-// selects its CTA shape (p = 1: 0 four CTAs per SM, 1 five)
+// selects its CTA shape at p = 1
 template <int P>
-cudaError_t stage_pair_launch(const StageArgs<3, P, float>& a, int grid, bool mortar, bool all_affine,
-                              cudaStream_t s, int v);
+cudaError_t stage_pair_launch(const StageArgs<3, P, float>& a, int grid, bool mortar, int shape, cudaStream_t s,
+                              int v);
 template <int P>
-int stage_pair_blocks_per_sm(int v);
+int stage_pair_blocks_per_sm(int v, int shape);
 template <int P>
-cudaError_t stage_pair_launch_batch(const StageArgs<3, P, float>& a, int grid, bool all_affine, cudaStream_t s);
+cudaError_t stage_pair_launch_batch(const StageArgs<3, P, float>& a, int grid, int shape, cudaStream_t s);
 
 template <int D, int P, int NS, typename Real>
 static int stage_blocks_per_sm_classic();
 
 template <int D, int P, int NS, typename Real>
-static int stage_blocks_per_sm_ns(int comp, int kernel) {
+static int stage_blocks_per_sm_ns(int comp, int kernel, int all_affine) {
   if constexpr (pair_shape<D, P, NS, Real>()) {
-    // kernel 2 (the five-CTA shape) exists at p = 1 only
+    // kernel 2 (the second CTA shape) exists at p = 1 only
     if (!comp && (kernel == 0 || (kernel == 2 && P == 1))) {
-      const int nb = stage_pair_blocks_per_sm<P>(kernel == 2);
+      const int nb = stage_pair_blocks_per_sm<P>(kernel == 2, all_affine);
       if (nb > 0) return nb;
     }
     if (kernel == 2) return 0;
@@ -173,11 +173,11 @@ static int stage_blocks_per_sm_classic() {
 }
 
 template <int D, int P, typename Real>
-static int stage_blocks_per_sm(int n, int comp, int kernel) {
+static int stage_blocks_per_sm(int n, int comp, int kernel, int all_affine) {
   switch (n) {
-    case 2: return stage_blocks_per_sm_ns<D, P, 2, Real>(comp, kernel);
-    case 4: return stage_blocks_per_sm_ns<D, P, 4, Real>(comp, kernel);
-    case 8: return stage_blocks_per_sm_ns<D, P, 8, Real>(comp, kernel);
+    case 2: return stage_blocks_per_sm_ns<D, P, 2, Real>(comp, kernel, all_affine);
+    case 4: return stage_blocks_per_sm_ns<D, P, 4, Real>(comp, kernel, all_affine);
+    case 8: return stage_blocks_per_sm_ns<D, P, 8, Real>(comp, kernel, all_affine);
   }
   return 0;  // n_seg other than 2, 4, 8 is not instantiated
 }
@@ -192,7 +192,7 @@ static cudaError_t stage_ns(const StageArgs<D, P, Real>& a, int slots, int comp,
     if (!comp && (kernel == 0 || kernel == 2)) {
       const int g = a.nL * a.nchunks < slots ? a.nL * a.nchunks : slots;
       if constexpr (P >= 1 && P <= 3)
-        return stage_pair_launch<P>(a, g, a.fluxmask != nullptr, all_affine != 0, s, kernel == 2 ? 1 : 0);
+        return stage_pair_launch<P>(a, g, a.fluxmask != nullptr, all_affine, s, kernel == 2 ? 1 : 0);
     }
   }
   if (a.fluxmask) return stage_mortar_launch<D, P, NS, Real>(a, grid, smem, comp, s);
@@ -498,7 +498,7 @@ template <int D, int P, typename Real>
 static int stage_batch_blocks_per_sm_p(int kernel, int all_affine) {
   if constexpr (D == 3 && std::is_same<Real, float>::value) {
     if constexpr (P >= 1 && P <= 3) {
-      if (kernel == 0) return stage_pair_blocks_per_sm<P>(0);
+      if (kernel == 0) return stage_pair_blocks_per_sm<P>(0, all_affine);
     }
     constexpr int YS = stage_rows<D, P, Real>(8);
     const size_t smem = stage_smem<D, P, Real>(8, YS);
@@ -524,7 +524,7 @@ static cudaError_t launch_stage_batch_p(const RtStage& common, const void* membe
     a.istart = istart;
     a.nmem = nmem;
     if constexpr (P >= 1 && P <= 3) {
-      if (common.kernel == 0) return stage_pair_launch_batch<P>(a, grid, common.all_affine != 0, s);
+      if (common.kernel == 0) return stage_pair_launch_batch<P>(a, grid, common.all_affine, s);
     }
     constexpr int YS = stage_rows<D, P, Real>(8);
     const size_t smem = stage_smem<D, P, Real>(8, YS);
@@ -674,12 +674,12 @@ static cudaError_t launch_guard_batch_p(const void* members, const int* bstart, 
     return cudaErrorInvalidValue;                                                           \
   }                                                                                         \
   template <>                                                                               \
-  int stage_occupancy<DIM, REAL>(int p, int n, int comp, int kernel) {                      \
+  int stage_occupancy<DIM, REAL>(int p, int n, int comp, int kernel, int all_affine) {      \
     switch (p) {                                                                            \
-      case 0: return stage_blocks_per_sm<DIM, 0, REAL>(n, comp, kernel);                    \
-      case 1: return stage_blocks_per_sm<DIM, 1, REAL>(n, comp, kernel);                    \
-      case 2: return stage_blocks_per_sm<DIM, 2, REAL>(n, comp, kernel);                    \
-      case 3: return stage_blocks_per_sm<DIM, 3, REAL>(n, comp, kernel);                    \
+      case 0: return stage_blocks_per_sm<DIM, 0, REAL>(n, comp, kernel, all_affine);        \
+      case 1: return stage_blocks_per_sm<DIM, 1, REAL>(n, comp, kernel, all_affine);        \
+      case 2: return stage_blocks_per_sm<DIM, 2, REAL>(n, comp, kernel, all_affine);        \
+      case 3: return stage_blocks_per_sm<DIM, 3, REAL>(n, comp, kernel, all_affine);        \
     }                                                                                       \
     return 0;                                                                               \
   }                                                                                         \

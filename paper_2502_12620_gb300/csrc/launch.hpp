@@ -23,7 +23,7 @@ struct RtStage {
   const void* gtr;
   const void* hcell;
   const unsigned char* affine;
-  int all_affine;  // every leaf affine
+  int all_affine;  // what every leaf is: 1 affine, 2 affine and axis-aligned, 0 neither
   const void* ameta;
   const int* kind;
   const int* nbr;
@@ -166,6 +166,6 @@ cudaError_t launch_guard_batch(int p, const void* members, const int* bstart, co
                                long long blocks, cudaStream_t s);
 // resident stage CTAs per SM (0: does not fit)
 template <int D, typename Real>
-int stage_occupancy(int p, int n, int comp, int kernel);
+int stage_occupancy(int p, int n, int comp, int kernel, int all_affine);
 
 }  // namespace dgf

@@ -151,18 +151,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 __device__ __forceinline__ void reload_fence() { asm volatile("" ::: "memory"); }
 
 // ------------------------------------------------------------- Euler, x2
-// F . a for a pair of states (Eq. (2)); also returns v.a, p and 1/rho
-__device__ __forceinline__ void flux2(const float2 (&u)[5], const float2 (&a)[3], float2 gm1, float2 (&F)[5],
-                                      float2& vn, float2& pr) {
+// AX >= 0: the area vector a has the one component AX (axis-aligned blocks);
+// the terms left out are exact zeros.
+template <int AX>
+__device__ __forceinline__ float2 dot2(const float2 (&u)[5], const float2 (&a)[3]) {
+  if constexpr (AX >= 0) return mul(u[1 + AX], a[AX]);
+  return fma2(u[3], a[2], fma2(u[2], a[1], mul(u[1], a[0])));
+}
+// F . a for a pair of states (Eq. (2))
+template <int AX>
+__device__ __forceinline__ void flux2(const float2 (&u)[5], const float2 (&a)[3], float2 gm1, float2 (&F)[5]) {
   const float2 ri = rcp2(u[0]);
-  const float2 mn = fma2(u[3], a[2], fma2(u[2], a[1], mul(u[1], a[0])));
+  const float2 mn = dot2<AX>(u, a);
   const float2 ke = fma2(u[3], u[3], fma2(u[2], u[2], mul(u[1], u[1])));
-  vn = mul(mn, ri);
-  pr = mul(gm1, fma2(mul(ke, ri), f2(-0.5f), u[4]));
+  const float2 vn = mul(mn, ri);
+  const float2 pr = mul(gm1, fma2(mul(ke, ri), f2(-0.5f), u[4]));
   F[0] = mn;
-  F[1] = fma2(u[1], vn, mul(pr, a[0]));
-  F[2] = fma2(u[2], vn, mul(pr, a[1]));
-  F[3] = fma2(u[3], vn, mul(pr, a[2]));
+#pragma unroll
+  for (int j = 0; j < 3; ++j) F[1 + j] = AX < 0 || AX == j ? fma2(u[1 + j], vn, mul(pr, a[j])) : mul(u[1 + j], vn);
   F[4] = mul(add(u[4], pr), vn);
 }
 
@@ -170,13 +176,12 @@ __device__ __forceinline__ void flux2(const float2 (&u)[5], const float2 (&a)[3]
 // once; a = area vector from L to R.  Both physical fluxes are summed into
 // the result term by term (fewer live registers than forming F(U_L) and
 // F(U_R) first).  A NaN wave speed (negative density or pressure)
-// propagates into the flux, as in lf_flux.
-// an = |a|.
+// propagates into the flux, as in lf_flux.  an = |a|.
+template <int AX>
 __device__ __forceinline__ void lf2(const float2 (&uL)[5], const float2 (&uR)[5], const float2 (&a)[3], float2 an,
                                     float2 gam, float2 gm1, float2 (&Fh)[5]) {
   const float2 riL = rcp2(uL[0]), riR = rcp2(uR[0]);
-  const float2 mnL = fma2(uL[3], a[2], fma2(uL[2], a[1], mul(uL[1], a[0])));
-  const float2 mnR = fma2(uR[3], a[2], fma2(uR[2], a[1], mul(uR[1], a[0])));
+  const float2 mnL = dot2<AX>(uL, a), mnR = dot2<AX>(uR, a);
   const float2 keL = fma2(uL[3], uL[3], fma2(uL[2], uL[2], mul(uL[1], uL[1])));
   const float2 keR = fma2(uR[3], uR[3], fma2(uR[2], uR[2], mul(uR[1], uR[1])));
   const float2 vL = mul(mnL, riL), vR = mul(mnR, riR);
@@ -189,9 +194,10 @@ __device__ __forceinline__ void lf2(const float2 (&uL)[5], const float2 (&uR)[5]
   const float2 pp = add(pL, pR);
   Fh[0] = mul(h, fma2(al, sub(uL[0], uR[0]), add(mnL, mnR)));
 #pragma unroll
-  for (int jx = 0; jx < 3; ++jx)
-    Fh[1 + jx] = mul(h, fma2(al, sub(uL[1 + jx], uR[1 + jx]),
-                             fma2(uL[1 + jx], vL, fma2(uR[1 + jx], vR, mul(pp, a[jx])))));
+  for (int j = 0; j < 3; ++j) {
+    const float2 R = AX < 0 || AX == j ? fma2(uR[1 + j], vR, mul(pp, a[j])) : mul(uR[1 + j], vR);
+    Fh[1 + j] = mul(h, fma2(al, sub(uL[1 + j], uR[1 + j]), fma2(uL[1 + j], vL, R)));
+  }
   Fh[4] = mul(h, fma2(al, sub(uL[4], uR[4]), fma2(add(uL[4], pL), vL, mul(add(uR[4], pR), vR))));
 }
 
@@ -201,7 +207,7 @@ __device__ __forceinline__ float2 norm2(const float2 (&a)[3]) {
 
 // The same for one face point.  split: with the two sides' fluxes rounded
 // before they are added and 1/2 |m|^2 / rho in one rounding, as lf_flux does;
-// the block's upper x face keeps those roundings, so that an affine forest's
+// the block's upper x face keeps those roundings, so that an affine block's
 // states stay the same bit for bit.
 __device__ __forceinline__ void lf1(const float (&uL)[5], const float (&uR)[5], const float (&a)[3], float an, float gam,
                                     float gm1, bool split, float (&Fh)[5]) {
@@ -298,14 +304,36 @@ struct LineGeo2 {
   }
 };
 
+// J dxi_DIR/dx of a pair of cells at one point (a face: xi[DIR] = -1 or 1),
+// from the tangents along the other two axes; half the work of a LineGeo2.
+// The face normals take this and the volume points LineGeo2 afterwards, so
+// that a line's metric is not held in registers across the face flux.
+template <int DIR>
+__device__ __forceinline__ void face_row2(const float* __restrict__ G, int cl, const float (&xi)[3], float2 (&Ja)[3],
+                                          int stride = 64) {
+  constexpr int i1 = (DIR + 1) % 3, i2 = (DIR + 2) % 3;
+  float2 t1[3], t2[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    auto X = [&](int c) { return lds2(G + ((c - 1) * 3 + j) * stride + cl); };
+    const float2 mix = fma2(X(7), f2(xi[DIR]), X((1 << i1) | (1 << i2)));
+    t1[j] = fma2(mix, f2(xi[i2]), fma2(X((1 << i1) | (1 << DIR)), f2(xi[DIR]), X(1 << i1)));
+    t2[j] = fma2(mix, f2(xi[i1]), fma2(X((1 << i2) | (1 << DIR)), f2(xi[DIR]), X(1 << i2)));
+  }
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+    Ja[j] = sub(mul(t1[j1], t2[j2]), mul(t1[j2], t2[j1]));
+  }
+}
+
 // barrier among the N warps of a group (hardware barriers 1 .. 2 N)
 template <int THREADS>
 __device__ __forceinline__ void group_sync(int id) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(THREADS) : "memory");
 }
 
-// V selects the CTA shape at p = 1 (0: four CTAs per SM, 1: five); one
-// shape at p = 2 and 3
+// V selects the CTA shape at p = 1; one shape at p = 2 and 3
 template <int P, int V = 0>
 struct PairCfg {
   static constexpr int N = P + 1, Q = N * N * N, NFP = N * N, NV = 5;
@@ -324,29 +352,38 @@ struct PairCfg {
   static constexpr bool UNREG = P == 1 && V == 0;
   // variables of the carried z-face flux that wait for the z lines in shared
   // memory instead of in registers: what is free beside the layers
-  static constexpr int park(bool aff) { return aff ? (P == 2 ? 4 : 5) : (P == 2 || V ? 0 : 5); }
+  static constexpr int park(bool aff) { return aff && P == 2 ? 4 : 5; }
   // shared memory: ST state layers, the residual layer, 2 geometry layers of
   // a curved block, the parked fluxes
   static constexpr size_t smem(bool aff) {
     return (size_t)((ST + 1) * ROWS * 64 + (aff ? 0 : 2 * NG * 64) + park(aff) * 2 * NT) * sizeof(float);
   }
-  // resident CTAs per SM: shared memory allows 2 at p = 2 (about 114 KB each)
-  // and 5 at p = 1; at p = 1 four CTAs leave 128 registers per thread (16
-  // warps, 4 per scheduler), five only 96 (more warps, more spills: the
-  // autotuner times both); at p = 3 one CTA of 16 warps with 128 registers
-  static constexpr int MINB = P <= 1 ? (V ? 5 : 4) : P == 2 ? 2 : 1;
+  // Resident CTAs per SM.  Affine blocks: 2 at p = 2 (about 112 KB of shared
+  // memory each, 96 registers), at p = 1 four (128 registers) or five (V = 1,
+  // 96 registers, more warps; the autotuner times both), one of 16 warps with
+  // 128 registers at p = 3.  Curved blocks hold the metric of a line too and
+  // spilled 740 to 1020 bytes in these shapes, so they take fewer CTAs with
+  // 168 registers: one at p = 2, three (V = 1: two) at p = 1.  Per stage, 71
+  // curved blocks p = 2 59.5 -> 50.2 us, 216 blocks 144 -> 133 us, p = 1 49.4
+  // -> 38.8 us.
+  static constexpr int minb(bool aff) {
+    return P <= 1 ? (aff ? (V ? 5 : 4) : (V ? 2 : 3)) : P == 2 ? (aff ? 2 : 1) : 1;
+  }
 };
 
 }  // namespace pairk
 
-// AFF: every block of the forest is affine (no per-cell geometry is read;
-// the curved code paths are not compiled into this instantiation)
+// GEO: 0 blocks of any shape, 1 every block of the forest affine (no per-cell
+// geometry is read, the curved code is not compiled), 2 every block affine
+// and axis-aligned (one component of each area vector)
 // BATCH: one launch for every forest of a batch (A.members; the tables and
 // stage coefficients of A are common to all of them).
-template <int P, bool MORTAR, bool AFF, bool BATCH = false, int V = 0>
-__global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>::MINB)
+template <int P, bool MORTAR, int GEO, bool BATCH = false, int V = 0>
+__global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>::minb(GEO != 0))
     k_stage_pair(const __grid_constant__ StageArgs<3, P, float> A, const __grid_constant__ pairk::PairTab<P + 1> T2) {
   static_assert(!(BATCH && MORTAR), "batches run without the mortar repair");
+  constexpr bool AFF = GEO != 0, DIAG = GEO == 2;
+  constexpr int AX = DIAG ? 0 : -1, AY = DIAG ? 1 : -1, AZ = DIAG ? 2 : -1;
   using namespace pairk;
   using C = PairCfg<P, V>;
   constexpr int N = C::N, Q = C::Q, NFP = C::NFP, NV = 5, ROWS = C::ROWS, NG = C::NG;
@@ -569,10 +606,8 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
 #pragma unroll
           for (int jj = 0; jj < 3; ++jj) Ja[jj] = f2(sam[6 + jj]);
         } else {
-          LineGeo2<2> lg;
-          const float xi[3] = {xa, xb, 0.f};
-          lg.init(Gs + (L & 1) * NG * LAY, cl, xi);
-          lg.at(-1.f, Ja);
+          const float xi[3] = {xa, xb, -1.f};
+          face_row2<2>(Gs + (L & 1) * NG * LAY, cl, xi, Ja);
         }
       } else {
         const float* Ul = pUb() + (k0 - 1) * LAY + cl;  // the layer below, from memory
@@ -588,13 +623,11 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
 #pragma unroll
           for (int jj = 0; jj < 3; ++jj) Ja[jj] = f2(sam[6 + jj]);
         } else {
-          LineGeo2<2> lg;
-          const float xi[3] = {xa, xb, 0.f};
-          lg.init(pGeo() + (k0 - 1) * LAY, cl, xi, nc);
-          lg.at(1.f, Ja);
+          const float xi[3] = {xa, xb, 1.f};
+          face_row2<2>(pGeo() + (k0 - 1) * LAY, cl, xi, Ja, nc);
         }
       }
-      lf2(tl, tm, Ja, aff ? f2(san[2]) : norm2(Ja), gam, gm1, Fbot);
+      lf2<AZ>(tl, tm, Ja, aff ? f2(san[2]) : norm2(Ja), gam, gm1, Fbot);
       if (MORTAR && k0 == 0 && (fmask & 16)) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) Fbot[v] = tl[v];  // the z- face flux itself
@@ -694,7 +727,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
           uL[v] = up ? in[v] : ev[v];
           uR[v] = up ? ev[v] : in[v];
         }
-        lf1(uL, uR, Je, an, A.gamma, A.gamma - 1.f, AFF && ef == 1, Fe);
+        lf1(uL, uR, Je, an, A.gamma, A.gamma - 1.f, ef == 1, Fe);
         const bool given = MORTAR && ((fmask >> ef) & 1);  // the outer value is the flux itself
 #pragma unroll
         for (int v = 0; v < NV; ++v) ev[v] = given ? ev[v] : Fe[v];
@@ -717,17 +750,14 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
             tp[v] = fma2(T2.lp[qx], x, tp[v]);
           }
         }
-        // face normals at xi_x = -1 (both cells); the metric along the line is
-        // evaluated again for the volume points below
+        // face normals at xi_x = -1 (both cells)
         float2 Jm[3];
         if (aff) {
 #pragma unroll
           for (int jj = 0; jj < 3; ++jj) Jm[jj] = f2(sam[jj]);
         } else {
-          LineGeo2<0> lg;
-          const float xi[3] = {0.f, xa, xb};
-          lg.init(Gc, cl, xi);
-          lg.at(-1.f, Jm);
+          const float xi[3] = {-1.f, xa, xb};
+          face_row2<0>(Gc, cl, xi, Jm);
         }
         reload_fence();
         // left face of each cell of the pair: (face i0, face i0+1); the
@@ -741,7 +771,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
             const float nb = __shfl_up_sync(0xffffffffu, tp[v].y, 1);
             uL[v] = make_float2(m == 0 ? tm[v].x : nb, tp[v].x);
           }
-          lf2(uL, tm, Jm, aff ? f2(san[0]) : norm2(Jm), gam, gm1, Fl);
+          lf2<AX>(uL, tm, Jm, aff ? f2(san[0]) : norm2(Jm), gam, gm1, Fl);
         }
         // right faces: the next pair's left face; the block's x+ face on m == 3
 #pragma unroll
@@ -765,7 +795,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
         }
 #pragma unroll
         for (int jj = 0; jj < N; ++jj) {
-          float2 uq[NV], Jq[3], G[NV], vn, pr;
+          float2 uq[NV], Jq[3], G[NV];
 #pragma unroll
           for (int v = 0; v < NV; ++v) uq[v] = lds2(Uc + (v * Q + jj + N * fpX) * LAY + cl);
           if (aff) {
@@ -774,7 +804,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
           } else {
             lg.at(xq[jj], Jq);
           }
-          flux2(uq, Jq, gm1, G, vn, pr);
+          flux2<AX>(uq, Jq, gm1, G);
 #pragma unroll
           for (int qx = 0; qx < N; ++qx)
 #pragma unroll
@@ -810,10 +840,8 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
 #pragma unroll
           for (int jj = 0; jj < 3; ++jj) Jm[jj] = f2(sam[3 + jj]);
         } else {
-          LineGeo2<1> lg;
-          const float xi[3] = {xa, 0.f, xb};
-          lg.init(Gc, cl, xi);
-          lg.at(-1.f, Jm);
+          const float xi[3] = {xa, -1.f, xb};
+          face_row2<1>(Gc, cl, xi, Jm);
         }
         reload_fence();
         // bottom face of my row: against the row below; the block's y- and y+
@@ -826,7 +854,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
             const float2 nb = shfl_up2(tp[v], 4);
             uL[v] = j == 0 ? tm[v] : nb;
           }
-          lf2(uL, tm, Jm, aff ? f2(san[1]) : norm2(Jm), gam, gm1, Fb);
+          lf2<AY>(uL, tm, Jm, aff ? f2(san[1]) : norm2(Jm), gam, gm1, Fb);
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
@@ -854,7 +882,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
                             fma2(T2.lpwn[qy], Ft[v], lds2(Rs + (v * Q + fa + N * qy + NFP * fb) * LAY + cl)));
 #pragma unroll
         for (int jj = 0; jj < N; ++jj) {
-          float2 uq[NV], Jq[3], G[NV], vn, pr;
+          float2 uq[NV], Jq[3], G[NV];
 #pragma unroll
           for (int v = 0; v < NV; ++v) uq[v] = lds2(Uc + (v * Q + fa + N * jj + NFP * fb) * LAY + cl);
           if (aff) {
@@ -863,7 +891,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
           } else {
             lg.at(xq[jj], Jq);
           }
-          flux2(uq, Jq, gm1, G, vn, pr);
+          flux2<AY>(uq, Jq, gm1, G);
 #pragma unroll
           for (int qy = 0; qy < N; ++qy)
 #pragma unroll
@@ -927,13 +955,11 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
 #pragma unroll
             for (int jj = 0; jj < 3; ++jj) Ja[jj] = f2(sam[6 + jj]);
           } else {
-            LineGeo2<2> lg;
-            const float xi[3] = {xa, xb, 0.f};
-            lg.init(Gc, cl, xi);
-            lg.at(1.f, Ja);
+            const float xi[3] = {xa, xb, 1.f};
+            face_row2<2>(Gc, cl, xi, Ja);
           }
           reload_fence();
-          lf2(tp, th, Ja, aff ? f2(san[2]) : norm2(Ja), gam, gm1, Ft);
+          lf2<AZ>(tp, th, Ja, aff ? f2(san[2]) : norm2(Ja), gam, gm1, Ft);
           if (MORTAR && k == n - 1 && (fmask & 32)) {
 #pragma unroll
             for (int v = 0; v < NV; ++v) Ft[v] = th[v];  // the z+ face flux itself
@@ -968,7 +994,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
         }
 #pragma unroll
         for (int jj = 0; jj < N; ++jj) {
-          float2 uq[NV], Jq[3], G[NV], vn, pr;
+          float2 uq[NV], Jq[3], G[NV];
 #pragma unroll
           for (int v = 0; v < NV; ++v) uq[v] = lds2(Uc + (v * Q + fpZ + NFP * jj) * LAY + cl);
           if (aff) {
@@ -979,7 +1005,7 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
             lg.at(xq[jj], Jq);
             iJ[jj] = rcp2(lg.jac(Jq));
           }
-          flux2(uq, Jq, gm1, G, vn, pr);
+          flux2<AZ>(uq, Jq, gm1, G);
 #pragma unroll
           for (int qz = 0; qz < N; ++qz)
 #pragma unroll
@@ -1097,74 +1123,70 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
 // launch (grid = persistent CTAs, or one per work item) and resident CTAs
 // per SM, for the launch layer in kernels_inst.cuh; v = the CTA shape
 template <int P, int V>
-cudaError_t stage_pair_launch_v(const StageArgs<3, P, float>& a, int grid, bool mortar, bool all_affine,
-                                cudaStream_t s) {
+cudaError_t stage_pair_launch_v(const StageArgs<3, P, float>& a, int grid, bool mortar, int shape, cudaStream_t s) {
   using C = pairk::PairCfg<P, V>;
   const pairk::PairTab<P + 1> t2 = pairk::pair_tab<P + 1>(a.T);
   if (mortar) {
-    if (all_affine) k_stage_pair<P, true, true, false, V><<<grid, C::NT, C::smem(true), s>>>(a, t2);
-    else k_stage_pair<P, true, false, false, V><<<grid, C::NT, C::smem(false), s>>>(a, t2);
+    if (shape) k_stage_pair<P, true, 1, false, V><<<grid, C::NT, C::smem(true), s>>>(a, t2);
+    else k_stage_pair<P, true, 0, false, V><<<grid, C::NT, C::smem(false), s>>>(a, t2);
   } else {
-    if (all_affine) k_stage_pair<P, false, true, false, V><<<grid, C::NT, C::smem(true), s>>>(a, t2);
-    else k_stage_pair<P, false, false, false, V><<<grid, C::NT, C::smem(false), s>>>(a, t2);
+    if (shape == 2) k_stage_pair<P, false, 2, false, V><<<grid, C::NT, C::smem(true), s>>>(a, t2);
+    else if (shape) k_stage_pair<P, false, 1, false, V><<<grid, C::NT, C::smem(true), s>>>(a, t2);
+    else k_stage_pair<P, false, 0, false, V><<<grid, C::NT, C::smem(false), s>>>(a, t2);
   }
   return cudaGetLastError();
 }
 
+// shape: what every block of the forest is (GEO of k_stage_pair)
 template <int P>
-cudaError_t stage_pair_launch(const StageArgs<3, P, float>& a, int grid, bool mortar, bool all_affine,
-                              cudaStream_t s, int v) {
+cudaError_t stage_pair_launch(const StageArgs<3, P, float>& a, int grid, bool mortar, int shape, cudaStream_t s, int v) {
   if constexpr (P == 1) {
-    if (v) return stage_pair_launch_v<P, 1>(a, grid, mortar, all_affine, s);
+    if (v) return stage_pair_launch_v<P, 1>(a, grid, mortar, shape, s);
   }
-  return stage_pair_launch_v<P, 0>(a, grid, mortar, all_affine, s);
+  return stage_pair_launch_v<P, 0>(a, grid, mortar, shape, s);
 }
 
 // one launch over the forests of a batch (a.members); plain form, no mortar
 template <int P>
-cudaError_t stage_pair_launch_batch(const StageArgs<3, P, float>& a, int grid, bool all_affine, cudaStream_t s) {
+cudaError_t stage_pair_launch_batch(const StageArgs<3, P, float>& a, int grid, int shape, cudaStream_t s) {
   using C = pairk::PairCfg<P>;
   const pairk::PairTab<P + 1> t2 = pairk::pair_tab<P + 1>(a.T);
-  if (all_affine) k_stage_pair<P, false, true, true><<<grid, C::NT, C::smem(true), s>>>(a, t2);
-  else k_stage_pair<P, false, false, true><<<grid, C::NT, C::smem(false), s>>>(a, t2);
+  if (shape == 2) k_stage_pair<P, false, 2, true><<<grid, C::NT, C::smem(true), s>>>(a, t2);
+  else if (shape) k_stage_pair<P, false, 1, true><<<grid, C::NT, C::smem(true), s>>>(a, t2);
+  else k_stage_pair<P, false, 0, true><<<grid, C::NT, C::smem(false), s>>>(a, t2);
   return cudaGetLastError();
 }
 
-template <int P, bool MORTAR, bool AFF, bool BATCH = false, int V = 0>
+template <int P, bool MORTAR, int GEO, bool BATCH = false, int V = 0>
 int pair_blocks_per_sm_one() {
   using C = pairk::PairCfg<P, V>;
-  if (cudaFuncSetAttribute(k_stage_pair<P, MORTAR, AFF, BATCH, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)C::smem(AFF)) != cudaSuccess)
-    return 0;
+  auto* k = k_stage_pair<P, MORTAR, GEO, BATCH, V>;
+  const size_t smem = C::smem(GEO != 0);
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_stage_pair<P, MORTAR, AFF, BATCH, V>, C::NT, C::smem(AFF)) !=
-      cudaSuccess)
-    return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, C::NT, smem) != cudaSuccess) return 0;
   return nb;
 }
 
-// the fewest resident CTAs over the instantiations one forest may launch
-// (shape v; the batch instantiations have shape 0)
+// the fewest resident CTAs over the instantiations that a forest of this
+// shape may launch (CTA shape v; batches have shape 0)
+template <int P, int GEO, int V>
+int pair_blocks_per_sm() {
+  int o = pair_blocks_per_sm_one<P, false, GEO, false, V>();
+  auto least = [&](int x) { o = x < o ? x : o; };
+  least(pair_blocks_per_sm_one<P, true, GEO != 0, false, V>());
+  if constexpr (V == 0) least(pair_blocks_per_sm_one<P, false, GEO, true>());
+  return o;
+}
 template <int P>
-int stage_pair_blocks_per_sm(int v) {
-  int o[6];
-  if (P == 1 && v) {
-    o[0] = pair_blocks_per_sm_one<P, false, false, false, 1>();
-    o[1] = pair_blocks_per_sm_one<P, true, false, false, 1>();
-    o[2] = pair_blocks_per_sm_one<P, false, true, false, 1>();
-    o[3] = pair_blocks_per_sm_one<P, true, true, false, 1>();
-    o[4] = o[5] = o[0];
-  } else {
-    o[0] = pair_blocks_per_sm_one<P, false, false>();
-    o[1] = pair_blocks_per_sm_one<P, true, false>();
-    o[2] = pair_blocks_per_sm_one<P, false, true>();
-    o[3] = pair_blocks_per_sm_one<P, true, true>();
-    o[4] = pair_blocks_per_sm_one<P, false, false, true>();
-    o[5] = pair_blocks_per_sm_one<P, false, true, true>();
+int stage_pair_blocks_per_sm(int v, int shape) {
+  if constexpr (P == 1) {
+    if (v)
+      return shape == 2 ? pair_blocks_per_sm<P, 2, 1>() : shape ? pair_blocks_per_sm<P, 1, 1>()
+                                                                : pair_blocks_per_sm<P, 0, 1>();
   }
-  int lo = o[0];
-  for (int i = 1; i < 6; ++i) lo = o[i] < lo ? o[i] : lo;
-  return lo;
+  return shape == 2 ? pair_blocks_per_sm<P, 2, 0>() : shape ? pair_blocks_per_sm<P, 1, 0>()
+                                                            : pair_blocks_per_sm<P, 0, 0>();
 }
 
 }  // namespace dgf
