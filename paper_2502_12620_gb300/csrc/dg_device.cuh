@@ -396,6 +396,7 @@ struct GuardArgs {
   const Real* __restrict__ ctr;    // [op][2^D M][NFP]: the same operator followed by my face trace
   const int* __restrict__ fine_list;  // [nfine] leaf * 2D + face of every finer-neighbour face
   int nfine;
+  int fine_warps;                     // time step: one warp per guard cell of a finer face, else one block
   const int* __restrict__ trd;        // [b][f][8] face-trace descriptors (kinds 0, 1, 3), see k_guard_trace
   const int* __restrict__ tlist;      // [ntr] leaf * 2D + face of the faces to trace, null: every face
   int ntr;
@@ -1644,13 +1645,19 @@ __device__ __forceinline__ void guard_trace_block(const GuardArgs<D, P, Real>& A
     for (int j = 0; j < NFP; ++j) out_trace[(size_t)j * nt] = tr[j];
     return;
   }
-  // ---- finer faces: one block per (finer face, guard cell t), all vars;
-  // warp e applies fine child e's columns of the trace operator
+  // ---- finer faces: the trace operator's columns of each fine child, the
+  // children's partial sums added in order.  With few guard cells one block
+  // takes a cell, a warp per child (the shortest chain); with many one warp
+  // takes a cell and goes through the children, the next one's values loaded
+  // while one is summed: 680 blocks at p = 1 have 12,400 such cells, and blocks
+  // of 20 busy lanes in 256 took 38 us a stage for them.
   constexpr int NPAIR = NV * NFP;
+  constexpr int ROUNDS = (NPAIR + 31) / 32, VPL = (NV * Q + 31) / 32;
   __shared__ Real sv[NW][NV][Q];
   __shared__ Real pv[NW][NPAIR];
-  const unsigned item = bid;
-  const int lane = threadIdx.x & 31, e = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned item = A.fine_warps ? bid * NW + wid : bid;
+  if (item >= (unsigned)A.nfine << lnt) return;  // whole warps, and only with a warp per cell
   const int t = (int)(item & (unsigned)(nt - 1));
   const int bf = A.fine_list[item >> lnt];
   const int b = bf / (2 * D), f = bf % (2 * D);
@@ -1676,38 +1683,75 @@ __device__ __forceinline__ void guard_trace_block(const GuardArgs<D, P, Real>& A
   }
   h[b2] = s2 == 0 ? 0 : n - 1;
   const int fine = A.nbr[bf * 4 + sub];
-  int c = 0, st = 1;
-  for (int ax = 0; ax < D; ++ax) {
-    const int cN = (2 * h[ax]) / n;
-    c += (2 * h[ax] + ((e >> ax) & 1) - cN * n) * st;
-    st *= n;
-  }
-  for (int i = lane; i < NV * Q; i += 32) {
-    const int v = i / Q, q = i % Q;
-    sv[e][v][q] = S((((size_t)fine * NV + v) * Q + q) * nc + c);
-  }
-  __syncwarp();
   const int co = A.copoff[bf];  // first operator << 1 | one operator shared by every guard cell
-  const Real* op = A.ctr + ((size_t)(co >> 1) + ((co & 1) ? 0 : t)) * KC * NFP + (size_t)e * Q * NFP;
-  for (int pr = lane; pr < NPAIR; pr += 32) {
+  const Real* opt = A.ctr + ((size_t)(co >> 1) + ((co & 1) ? 0 : t)) * KC * NFP;
+  // cell of fine child e under the guard cell
+  auto child = [&](int e) {
+    int c = 0, st = 1;
+    for (int ax = 0; ax < D; ++ax) {
+      const int cN = (2 * h[ax]) / n;
+      c += (2 * h[ax] + ((e >> ax) & 1) - cN * n) * st;
+      st *= n;
+    }
+    return c;
+  };
+  // child e's part of pair pr from its values in row r of sv
+  auto part = [&](int e, int r, int pr) -> Real {
+    const Real* op = opt + (size_t)e * Q * NFP;
     const int v = pr / NFP, fp = pr % NFP;
     Real acc0 = Real(0), acc1 = Real(0);
     // every load of the operator's column before the sums: one trip to L2
 #pragma unroll(Q <= 27 ? Q / 2 : 8)
     for (int q = 0; q + 1 < Q; q += 2) {
-      acc0 += __ldg(&op[(size_t)q * NFP + fp]) * sv[e][v][q];
-      acc1 += __ldg(&op[(size_t)(q + 1) * NFP + fp]) * sv[e][v][q + 1];
+      acc0 += __ldg(&op[(size_t)q * NFP + fp]) * sv[r][v][q];
+      acc1 += __ldg(&op[(size_t)(q + 1) * NFP + fp]) * sv[r][v][q + 1];
     }
-    if (Q & 1) acc0 += __ldg(&op[(size_t)(Q - 1) * NFP + fp]) * sv[e][v][Q - 1];
-    pv[e][pr] = acc0 + acc1;
+    if (Q & 1) acc0 += __ldg(&op[(size_t)(Q - 1) * NFP + fp]) * sv[r][v][Q - 1];
+    return acc0 + acc1;
+  };
+  const size_t src = (size_t)fine * NV * Q;
+  if (A.fine_warps) {
+    Real x[VPL], tot[ROUNDS];
+    auto load = [&](int e) {
+      const int c = child(e);
+#pragma unroll
+      for (int i = 0; i < VPL; ++i)
+        if (lane + 32 * i < NV * Q) x[i] = S((src + lane + 32 * i) * nc + c);
+    };
+    load(0);
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) tot[r] = Real(0);
+#pragma unroll 1
+    for (int e = 0; e < NW; ++e) {
+      __syncwarp();  // the child before is summed
+#pragma unroll
+      for (int i = 0; i < VPL; ++i)
+        if (lane + 32 * i < NV * Q) (&sv[wid][0][0])[lane + 32 * i] = x[i];
+      __syncwarp();
+      if (e + 1 < NW) load(e + 1);
+#pragma unroll
+      for (int r = 0; r < ROUNDS; ++r)
+        if (lane + 32 * r < NPAIR) tot[r] += part(e, wid, lane + 32 * r);
+    }
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+      const int pr = lane + 32 * r;
+      if (pr < NPAIR) A.out[(((size_t)b * 2 * D + f) * NPAIR + pr) * nt + t] = tot[r];
+    }
+    return;
   }
+  {
+    const int c = child(wid);
+    for (int i = lane; i < NV * Q; i += 32) (&sv[wid][0][0])[i] = S((src + i) * nc + c);
+  }
+  __syncwarp();
+  for (int pr = lane; pr < NPAIR; pr += 32) pv[wid][pr] = part(wid, wid, pr);
   __syncthreads();
   for (int pr = threadIdx.x; pr < NPAIR; pr += NTH) {
     Real acc = Real(0);
 #pragma unroll
     for (int ee = 0; ee < NW; ++ee) acc += pv[ee][pr];
-    const int v = pr / NFP, fp = pr % NFP;
-    A.out[((((size_t)b * 2 * D + f) * NV + v) * NFP + fp) * nt + t] = acc;
+    A.out[(((size_t)b * 2 * D + f) * NPAIR + pr) * nt + t] = acc;
   }
 }
 

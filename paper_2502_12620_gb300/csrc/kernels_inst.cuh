@@ -265,9 +265,19 @@ static cudaError_t stage_p(const RtStage& r, cudaStream_t s) {
   return cudaErrorInvalidConfiguration;
 }
 
+// Guard cells of finer faces: a block each while all of them fit the GPU at
+// once (eight 256-thread blocks an SM), a warp each beyond two such rounds.
+static inline bool fine_by_warps(const RtGuard& r, int nt) { return (long long)r.nfine * nt > 2 * 8 * 152; }
+template <int D>
+static int fine_blocks(const RtGuard& r) {
+  const int nt = D == 3 ? r.n * r.n : r.n;
+  return fine_by_warps(r, nt) ? (r.nfine * nt + (1 << D) - 1) >> D : r.nfine * nt;
+}
+
 template <int D, int P, typename Real>
 static GuardArgs<D, P, Real> make_guard_args(const RtGuard& r) {
   GuardArgs<D, P, Real> a;
+  a.fine_warps = fine_by_warps(r, D == 3 ? r.n * r.n : r.n);
   a.nL = r.nL;
   a.n = r.n;
   a.mode = r.mode;
@@ -313,7 +323,7 @@ static cudaError_t guard_p(const RtGuard& r, cudaStream_t s) {
     const size_t items = (size_t)a.ntr * (D + 2) * nt;
     if (items >= ((size_t)1 << 32)) return cudaErrorInvalidConfiguration;  // the kernel indexes in 32 bits
     const size_t ntb = (items + NTH - 1) / NTH;
-    const int nfb = r.nfine * nt;
+    const int nfb = fine_blocks<D>(r);
     if (ntb + nfb == 0) return cudaSuccess;  // every face is traced by the stage kernel
     const bool comp = std::is_same<Real, float>::value && r.comp;
     if constexpr (std::is_same<Real, float>::value) {
@@ -490,7 +500,7 @@ static long long guard_blocks_p(const RtGuard& r, int* nfb) {
   constexpr int NTH = 32 << D;
   const int nt = D == 3 ? r.n * r.n : r.n;
   const size_t items = (size_t)(r.tlist ? r.ntr : r.nL * 2 * D) * (D + 2) * nt;
-  *nfb = r.nfine * nt;
+  *nfb = fine_blocks<D>(r);
   return (long long)((items + NTH - 1) / NTH) + *nfb;
 }
 
