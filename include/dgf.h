@@ -275,10 +275,11 @@ dgf_status dgf_status_word(dgf_forest* f, int32_t* status, int reset);
 dgf_status dgf_tuning(const dgf_forest* f, int32_t* zchunk, int32_t* resident_ctas);
 
 /* Which stage kernel the forest's time step launches (host value, no sync):
- * 0 = the cell-pair FP32 kernel (3D forests of 8^3-cell blocks at p = 1, 2
- * in plain FP32: f32x2 arithmetic on cell pairs, TMA-staged layers; four
- * CTAs per SM at p = 1), 1 = the general layer-sweep kernel, 2 = the
- * cell-pair kernel in its five-CTA shape (p = 1 only: more warps, fewer
+ * 0 = the cell-pair FP32 kernel (3D forests of 8^3-cell blocks at p = 1..3
+ * in plain FP32: f32x2 arithmetic on cell pairs, TMA-staged layers, traces
+ * read from the neighbours; four CTAs per SM at p = 1), 1 = the general
+ * layer-sweep kernel, 2 = the cell-pair kernel in its second CTA shape
+ * (p = 1 only; affine forests: five CTAs per SM, more warps with fewer
  * registers).  The first dgf_rk_step of a 3D forest times every kernel that
  * applies and keeps the fastest (the z-chunk length and the grid are tuned
  * with it); DGF_STAGE_KERNEL=pair|pair5|classic in the environment pins the
@@ -298,7 +299,8 @@ dgf_status dgf_stage_grid(const dgf_forest* f, int32_t* per_item);
 /* Kernel timing: when on, rk_step launches stage by stage (no graph) with
  * CUDA events around every kernel; dgf_kernel_times synchronises and returns
  * summed milliseconds and kernel launch counts for the classes 0 = dt,
- * 1 = guard (with the mortar passes and the limiter), 2 = stage, then resets
+ * 1 = guard (with the mortar passes and the limiter; none where the stage
+ * kernel traces every face), 2 = stage, then resets
  * the sums. */
 dgf_status dgf_set_timing(dgf_forest* f, int on);
 dgf_status dgf_kernel_times(dgf_forest* f, double* ms, int64_t* launches, int n_classes);

@@ -445,7 +445,9 @@ __host__ __device__ constexpr size_t stage_smem(int n, int rows) {
   size_t fx = (size_t)NV * NFP * (n + 1) * rows, fy = (size_t)NV * NFP * (rows + 1) * n;
   size_t fz = D == 3 ? (size_t)NV * NFP * ncl : 0;
   size_t ri = sizeof(Real) == 8 ? Q * ncl : 0;  // 1 / rho, FP64
-  return (us + rs + fx + fy + fz + ri) * sizeof(Real);
+  // FP64 in 2D: the y lines' own residual and 1/J
+  size_t ry = sizeof(Real) == 8 && D == 2 ? rs + Q * ncl : 0;
+  return (us + rs + fx + fy + fz + ri + ry) * sizeof(Real);
 }
 
 // rows of a layer one work item sweeps: the whole layer when its buffers fit
@@ -617,6 +619,10 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
   __shared__ Real sx[N];
   __shared__ Real sam[D * D + 1];
   constexpr bool SHRI = sizeof(Real) == 8;
+  // FP64 in 2D: x and y lines side by side on different warps (a slab has 48
+  // of each at p = 2, two warps' worth: one after the other they left half of
+  // the SM's FP64 pipes idle), the y lines into a residual of their own
+  constexpr bool XY = SHRI && D == 2;
   constexpr int RSZ = NV * Q * NCL;
   Real* us = reinterpret_cast<Real*>(smem_raw);
   Real* rs = us + NV * Q * NCL;
@@ -625,6 +631,8 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
   Real* fz = fy + NV * NFP * (YR + 1) * n;
   Real* tb = fx;   // halo traces reuse the x-face buffer when it is free
   Real* rho1 = fz + (D == 3 ? NV * NFP * NCL : 0);  // [q][cell] 1 / rho (FP64)
+  Real* ry = rho1 + (SHRI ? Q * NCL : 0);           // [v][q][cell] the y lines' residual (XY)
+  Real* ijs = ry + (XY ? RSZ : 0);                  // [q][cell] 1 / J (XY)
   if (tid < N) sx[tid] = T.x[tid];
 
   Real lam_min = Real(3.0e38);
@@ -908,7 +916,56 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
       }
       __syncthreads();
       // ------------------------------------------- P3: x volume + lift (rs =)
-      for (int w = tid; w < NCL * NFP; w += nthr) {
+      constexpr int NXL = NCL * NFP;                    // x lines; beside them the y lines
+      constexpr int YOFF = (NXL + 31) / 32 * 32;
+      for (int w = tid; w < (XY ? YOFF + NXL : NXL); w += nthr) {
+        if constexpr (XY) {
+          if (w >= YOFF) {
+            const int c = (w - YOFF) % NCL, qx = (w - YOFF) / NCL;
+            const int i = c % n, j = c / n;
+            const Real xi[2] = {sx[qx], Real(0)};
+            LineGeo<2, 1, Real> lg;
+            if (!aff && !tab) lg.init(Gk + c, nc, xi);
+            Real F[N][NV];
+#pragma unroll
+            for (int qy = 0; qy < N; ++qy) {
+              const int q = qx + N * qy;
+              Real u[NV], Ja[2], Fq[NV], iJ;
+#pragma unroll
+              for (int v = 0; v < NV; ++v) u[v] = US(v, q, c);
+              if (aff) {
+                Ja[0] = sam[2];
+                Ja[1] = sam[3];
+                iJ = sam[4];
+              } else if (tab) {
+                Ja[0] = MET(2, q, cbase + c);
+                Ja[1] = MET(3, q, cbase + c);
+                iJ = MET(4, q, cbase + c);
+              } else {
+                lg.at(T.x[qy], Ja);
+                iJ = Real(1) / lg.jac(Ja);
+              }
+              ijs[q * NCL + c] = iJ;
+              flux_along<2, Real>(u, Ja, rho1[q * NCL + c], gm1, Fq);
+#pragma unroll
+              for (int v = 0; v < NV; ++v) F[qy][v] = Fq[v];
+            }
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+              const Real fm = FY(v, qx, j, i);
+              const Real fpl = FY(v, qx, j + 1, i);
+#pragma unroll
+              for (int qy = 0; qy < N; ++qy) {
+                Real s = Real(0);
+#pragma unroll
+                for (int jj = 0; jj < N; ++jj) s += T.Sh[qy][jj] * F[jj][v];
+                ry[(v * Q + qx + N * qy) * NCL + c] = s - T.lpw[qy] * fpl + T.lmw[qy] * fm;
+              }
+            }
+            continue;
+          }
+          if (w >= NXL) continue;
+        }
         const int c = w % NCL, fp = w / NCL;
         const int i = c % n, j = c / n;
         Real xi[D];
@@ -952,7 +1009,7 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
       __syncthreads();
       // ------------------------------------------- P4: y volume + lift (rs +=)
       //                                            and the halo trace above
-      constexpr int NY = NCL * NFP;
+      constexpr int NY = XY ? 0 : NCL * NFP;
       // halo items: HV consecutive cells with 16-byte loads and stores
       constexpr int HV = 16 / (int)sizeof(Real);
       constexpr int ny_total = NY + ((D == 3) ? NCL * NV * NFP / HV : 0);
@@ -1121,6 +1178,13 @@ __global__ void __launch_bounds__(StageCfg<P, Real>::NT, StageCfg<P, Real>::MINB
             const size_t gi = ((size_t)v * Q + q) * nc + cbase + c0;
             Real r[VEC], val[VEC];
             vload<VEC>(reinterpret_cast<const V*>(&RS(v, q, c0)), r);
+            if constexpr (XY) {
+              Real y[VEC], iJ[VEC];
+              vload<VEC>(reinterpret_cast<const V*>(&ry[(v * Q + q) * NCL + c0]), y);
+              vload<VEC>(reinterpret_cast<const V*>(&ijs[q * NCL + c0]), iJ);
+#pragma unroll
+              for (int e = 0; e < VEC; ++e) r[e] = (r[e] + y[e]) * iJ[e];
+            }
             if (A.mode == 1) {
 #pragma unroll
               for (int e = 0; e < VEC; ++e) val[e] = r[e];
@@ -1532,12 +1596,13 @@ __global__ void __launch_bounds__(32 << D) k_guard_fine(const GuardArgs<D, P, Re
 }
 
 // Guard traces for the time step (mode 1), one launch: the first
-// n_fine_blocks blocks run the finer-face combine (one block per finer face
-// and guard cell, all vars, one warp per fine child), the remaining blocks
-// compute the traces of same-level, coarser, outflow and prescribed-state
-// faces, one thread per (leaf, face, guard cell, var), from the host-built
-// face-trace descriptors (source cell and face points as affine functions
-// of my guard-cell and face-point digits).
+// n_fine_blocks blocks run the finer-face combine (one block or one warp per
+// finer face and guard cell, all vars), the remaining blocks compute the traces
+// of the other faces, one thread per (face, guard cell, var), from the
+// host-built face-trace descriptors (source cell and face points as affine
+// functions of my guard-cell and face-point digits): all of them for the
+// layer-sweep stage kernel, only level jumps and prescribed states (tlist) for
+// the cell-pair kernel, which traces the rest itself.
 // The body handles block `bid` of one forest's launch; k_guard_trace runs it
 // for one forest, k_guard_trace_batch for the forests of a batch (each
 // forest's blocks after the previous forests').

@@ -228,7 +228,7 @@ struct dgf_forest {
   Buf bstate;
   int slots = 0;            // resident CTAs of the chosen stage kernel
   // resident CTAs: [0] the cell-pair kernel where it applies, [1] k_stage,
-  // [2] the cell-pair kernel's five-CTA shape (p = 1; 0 elsewhere)
+  // [2] the cell-pair kernel's second CTA shape (p = 1; 0 elsewhere)
   int slots_k[3] = {0, 0, 0};
   int kernel = 0;           // stage kernel: 0 the cell-pair kernel where it applies, 1 k_stage
   bool grid_items = false;  // stage grid: one CTA per work item instead of the persistent CTAs
@@ -1205,7 +1205,7 @@ dgf_status autotune(dgf_forest* f) {
   std::vector<int> kernels;
   const char* ks = getenv("DGF_STAGE_KERNEL");
   // the cell-pair kernel is a candidate only where it applies (distinct
-  // slots), its five-CTA shape at p = 1; DGF_STAGE_KERNEL=pair|pair5|classic
+  // slots), its second CTA shape at p = 1; DGF_STAGE_KERNEL=pair|pair5|classic
   // keeps one
   const bool any = ks == nullptr;
   if ((any || strcmp(ks, "pair") == 0) && pair_applies(f) && f->slots_k[0] > 0) kernels.push_back(0);
