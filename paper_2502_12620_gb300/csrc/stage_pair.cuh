@@ -31,8 +31,8 @@
 // 4 to 5 warps a scheduler; registers and shared memory allow no more.
 // Per stage with the traces, before (a guard pass writing all traces, CTA
 // barriers; at p = 3 the layer-sweep kernel) and now: 4096 affine blocks,
-// p = 1: 326 + 80 -> 277 us; p = 2: 1040 + 258 -> 1143 us; 512 blocks, p = 3:
-// 514 + 76 -> 361 us.
+// p = 1: 326 + 80 -> 274 us; p = 2: 1040 + 258 -> 1130 us; 512 blocks, p = 3:
+// 514 + 76 -> 347 us.
 //
 // Per layer: x lines (volume flux, derivative, x faces, lift) -> residual
 // in shared memory; y lines (+= the same along y); z lines (+= along z, the
@@ -346,7 +346,8 @@ struct PairCfg {
   static constexpr int ST = P <= 2 ? 2 : 1;
   // U^n of a z line's points: loaded into registers before the combination
   // (p = 1 with 128 registers), else copied by TMA into the residual rows the
-  // warp has read.  Per stage at 4096 blocks, p = 1: 277 us in registers, 297
+  // warp has read.  Per stage at 4096 blocks (both sides
+  // before the axis-aligned instantiation), p = 1: 277 us in registers, 297
   // by TMA; p = 2: 1240 us (spilled registers; spills miss the small L1 that
   // the shared memory leaves), 1143 us by TMA; 512 blocks, p = 3: 406, 361 us.
   static constexpr bool UNREG = P == 1 && V == 0;
