@@ -1853,8 +1853,11 @@ __global__ void __launch_bounds__(128) k_mortar_fine(const GuardArgs<D, P, Real>
   const auto& T = A.T;
   const size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= (size_t)A.nmf * nt * NFP) return;
-  const int fp = (int)(w % NFP);
-  const int t = (int)((w / NFP) % nt);
+  // guard cells fastest: the trace slots and the cells' rows are read and
+  // written along them.  What bounds it is the latency of one thread's loads;
+  // 24 faces of 8^2 cells, p = 2: 14.0 us with face points fastest, 8.4 now.
+  const int t = (int)(w % nt);
+  const int fp = (int)((w / nt) % NFP);
   const int bf = A.mfine[w / ((size_t)NFP * nt)];
   const int b = bf / (2 * D), f = bf % (2 * D);
   const int a = f >> 1, s = f & 1;
@@ -1905,9 +1908,9 @@ __global__ void __launch_bounds__(128) k_mortar_coarse(const GuardArgs<D, P, Rea
   const int nt = D == 3 ? n * n : n;
   const size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= (size_t)A.nmc * nt * NV * NFP) return;
-  const int j = (int)(w % NFP);
-  const int v = (int)((w / NFP) % NV);
-  const int t = (int)((w / ((size_t)NFP * NV)) % nt);
+  const int t = (int)(w % nt);  // fastest, as above (24 faces: 5.7 -> 4.7 us)
+  const int j = (int)((w / nt) % NFP);
+  const int v = (int)((w / ((size_t)nt * NFP)) % NV);
   const int i = (int)(w / ((size_t)NFP * NV * nt));
   const Real* __restrict__ wt = A.mw + ((size_t)i * NFP + j) * NSUB * NFP;
   const long long* __restrict__ src = A.msrc + ((size_t)i * nt + t) * NSUB;
