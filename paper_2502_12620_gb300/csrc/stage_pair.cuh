@@ -502,8 +502,15 @@ __global__ void __launch_bounds__(pairk::PairCfg<P, V>::NT, pairk::PairCfg<P, V>
         if (A.ca != 0.f) prefetch_row_l2(un + (size_t)r * nc + k * LAY, LAY * sizeof(float));
       }
     };
+    // An affine block has none to copy, yet completes the phase: buffer and
+    // parity are taken from L, which every layer advances, so one that left
+    // its phase open would put the curved blocks behind it out of step.
     auto issue_geo = [&](int k, int s, const float* geo) {
-      if (aff || w != 0) return;
+      if (AFF || w != 0) return;
+      if (aff) {
+        if (lane == 0) mbar_arrive(&gfull[s]);
+        return;
+      }
       if (lane == 0) mbar_arrive_expect(&gfull[s], NG * LAY * sizeof(float));
       __syncwarp();
       if (lane < NG) {
