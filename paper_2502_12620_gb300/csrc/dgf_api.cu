@@ -209,6 +209,7 @@ struct dgf_forest {
       dtout, nodal, fine, affine, ameta, trd, tlist, met, fmet;
   int nfine = 0;
   int ntr = 0;  // faces of tlist: coarser neighbours and prescribed states
+  bool tables = false;  // met and fmet hold the metric of the current leaves
   // mortar treatment of level jumps (reading R15)
   bool mortar = false;
   Buf fluxmask, mfine, mcoarse, mw, msrc;
@@ -250,14 +251,6 @@ struct dgf_forest {
 
 namespace {
 
-void* dev_alloc(dgf_forest* f, size_t bytes) {
-  if (bytes == 0) bytes = 16;
-  if (f->has_alloc) return f->alloc.alloc(f->alloc.ctx, bytes, (void*)f->stream);
-  void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
-  return p;
-}
-
 void dev_free(dgf_forest* f, dgf_forest::Buf& b) {
   if (!b.ptr) return;
   if (f->has_alloc) {
@@ -270,6 +263,39 @@ void dev_free(dgf_forest* f, dgf_forest::Buf& b) {
   }
   b.ptr = nullptr;
   b.bytes = 0;
+}
+
+// captured time steps hold the pointers and choices they were captured with
+void drop_graphs(dgf_forest* f) {
+  if (f->graph) cudaGraphExecDestroy(f->graph);
+  if (f->graph_alt) cudaGraphExecDestroy(f->graph_alt);
+  f->graph = f->graph_alt = nullptr;
+  f->graph_valid = false;
+}
+
+void drop_metric(dgf_forest* f) {
+  f->tables = false;
+  if (!f->met.ptr && !f->fmet.ptr) return;
+  cudaStreamSynchronize(f->stream);
+  drop_graphs(f);
+  dev_free(f, f->met);
+  dev_free(f, f->fmet);
+}
+
+// The stage kernel can do without the metric tables, and nothing else of a
+// forest's memory can be done without: where an allocation does not fit they
+// are given back for it.
+void* dev_alloc(dgf_forest* f, size_t bytes) {
+  if (bytes == 0) bytes = 16;
+  for (;;) {
+    void* p = nullptr;
+    if (f->has_alloc) p = f->alloc.alloc(f->alloc.ctx, bytes, (void*)f->stream);
+    else if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
+    if (p) return p;
+    cudaGetLastError();  // a refused cudaMalloc
+    if (!f->met.ptr && !f->fmet.ptr) return nullptr;
+    drop_metric(f);
+  }
 }
 
 bool ensure(dgf_forest* f, dgf_forest::Buf& b, size_t bytes) {
@@ -415,6 +441,7 @@ dgf_status build_device(dgf_forest* f) {
     cudaStreamSynchronize(f->stream);  // buffers may be freed or reused below
   }
   f->nL = L;
+  f->tables = false;
   Forest::Tables T = F.tables();
 
   std::vector<int> kind(L * nf), nbr(L * nf * 4), orient(L * nf), qbits(L), copoff(L * nf, -1);
@@ -869,32 +896,6 @@ dgf_status build_device(dgf_forest* f) {
   if (!ensure(f, f->gtr, (size_t)L * nf * f->nv * f->NFP * nt * f->esize) ||
       !ensure(f, f->part, (size_t)L * nc * f->nv * sizeof(double)))
     return fail(DGF_ENOMEM, "scratch allocation failed");
-  // metric tables for FP64 forests with curved blocks, where memory allows
-  // (the stage kernel evaluates the metric itself without them)
-  if (f->precision == DGF_FP64 && !f->all_affine) {
-    const size_t cells = (size_t)L * nc;
-    if (ensure(f, f->met, cells * (d * d + 1) * M * sizeof(double)) &&
-        ensure(f, f->fmet, cells * d * d * f->NFP * sizeof(double))) {
-      RtMisc r{};
-      r.p = f->p;
-      r.nL = (int)L;
-      r.n = n;
-      r.T = f->tab;
-      r.geo = f->geo.ptr;
-      r.met = f->met.ptr;
-      r.fmet = f->fmet.ptr;
-      if ((st = cuda_check(d == 2 ? launch_metric<2, double>(r, f->stream) : launch_metric<3, double>(r, f->stream),
-                           "metric tables")))
-        return st;
-    } else {
-      cudaGetLastError();  // a refused cudaMalloc
-      dev_free(f, f->met);
-      dev_free(f, f->fmet);
-    }
-  } else {
-    dev_free(f, f->met);
-    dev_free(f, f->fmet);
-  }
   // resident stage CTAs, and the z-chunk length that balances the
   // persistent CTAs best (a chunk costs its layers plus ~0.3 layer of halo)
   {
@@ -940,16 +941,46 @@ dgf_status build_device(dgf_forest* f) {
   f->grid_items = grid_env(false);
   f->tuned = d != 3 || (getenv("DGF_ZCHUNK") != nullptr && getenv("DGF_STAGE_KERNEL") != nullptr &&
                         getenv("DGF_STAGE_GRID") != nullptr);
-  if (f->graph) {
-    cudaGraphExecDestroy(f->graph);
-    f->graph = nullptr;
-  }
-  if (f->graph_alt) {
-    cudaGraphExecDestroy(f->graph_alt);
-    f->graph_alt = nullptr;
-  }
-  f->graph_valid = false;
+  drop_graphs(f);
   return DGF_OK;
+}
+
+// Metric tables of an FP64 forest with curved blocks, where memory allows.
+// Last in a build, and in a regrid after the state has been carried over: they
+// take up to nine tenths of the state copies' size, and what is allocated
+// before them has to fit.
+dgf_status build_metric(dgf_forest* f) {
+  if (f->device < 0) return DGF_OK;
+  DeviceGuard dg(f->device);
+  if (f->precision != DGF_FP64 || f->all_affine) {
+    drop_metric(f);
+    return DGF_OK;
+  }
+  const int d = f->d;
+  const size_t cells = (size_t)f->nL * f->nc;
+  // (a refused second table gives the first one back)
+  if (!ensure(f, f->met, cells * (d * d + 1) * f->M * sizeof(double)) ||
+      !ensure(f, f->fmet, cells * d * d * f->NFP * sizeof(double)) || !f->met.ptr) {
+    drop_metric(f);
+    return DGF_OK;
+  }
+  RtMisc r{};
+  r.p = f->p;
+  r.nL = (int)f->nL;
+  r.n = f->n;
+  r.T = f->tab;
+  r.geo = f->geo.ptr;
+  r.met = f->met.ptr;
+  r.fmet = f->fmet.ptr;
+  dgf_status st = cuda_check(
+      d == 2 ? launch_metric<2, double>(r, f->stream) : launch_metric<3, double>(r, f->stream), "metric tables");
+  f->tables = st == DGF_OK;
+  return st;
+}
+
+dgf_status build_all(dgf_forest* f) {
+  const dgf_status st = build_device(f);
+  return st ? st : build_metric(f);
 }
 
 RtStage stage_args(dgf_forest* f, int src, int dst, double ca, double cb, int mode, int last) {
@@ -968,8 +999,8 @@ RtStage stage_args(dgf_forest* f, int src, int dst, double ca, double cb, int mo
   r.orient = (const int*)f->orient.ptr;
   r.qbits = (const int*)f->qbits.ptr;
   r.trd = (const int*)f->trd.ptr;
-  r.met = f->met.ptr;
-  r.fmet = f->fmet.ptr;
+  r.met = f->tables ? f->met.ptr : nullptr;
+  r.fmet = f->tables ? f->fmet.ptr : nullptr;
   r.U = f->U[src].ptr;
   r.Un = f->U[0].ptr;
   r.Uout = f->U[dst].ptr;
@@ -1419,7 +1450,7 @@ dgf_status dgf_forest_create(const dgf_forest_desc* desc, const dgf_allocator* a
       return fail(DGF_ECUDA, "device scalars");
     }
   }
-  dgf_status st = build_device(f);
+  dgf_status st = build_all(f);
   if (st) {
     std::string e = g_err;
     dgf_forest_destroy(f);
@@ -1466,11 +1497,7 @@ dgf_status dgf_set_stream(dgf_forest* f, void* stream) {
   if (f->own_stream) cudaStreamDestroy(f->stream);
   f->own_stream = false;
   f->stream = (cudaStream_t)stream;
-  if (f->graph) cudaGraphExecDestroy(f->graph);
-  if (f->graph_alt) cudaGraphExecDestroy(f->graph_alt);
-  f->graph = nullptr;
-  f->graph_alt = nullptr;
-  f->graph_valid = false;
+  drop_graphs(f);
   return DGF_OK;
 }
 
@@ -1587,7 +1614,7 @@ dgf_status dgf_set_boundary(dgf_forest* f, const int32_t* root_face_kind, const 
     if (!std::isfinite(state[v])) return fail(DGF_EINVAL, "non-finite boundary state");
   f->bctag = tags;
   f->bstate_h.assign(state, state + f->nv);
-  return build_device(f);
+  return build_all(f);
 }
 
 dgf_status dgf_leaf_count(const dgf_forest* f, int64_t* n) {
@@ -1880,10 +1907,7 @@ dgf_status dgf_set_limiter(dgf_forest* f, double eps) {
   DeviceGuard dg(f->device);
   cudaStreamSynchronize(f->stream);
   f->limiter = eps;
-  if (f->graph) cudaGraphExecDestroy(f->graph);
-  if (f->graph_alt) cudaGraphExecDestroy(f->graph_alt);
-  f->graph = f->graph_alt = nullptr;
-  f->graph_valid = false;
+  drop_graphs(f);
   return DGF_OK;
 }
 
@@ -1977,7 +2001,7 @@ static bool combine_op_cell(dgf_forest* f, const double* const* child_coef, doub
 // state buffer is kept until the transfer kernel has run.
 static dgf_status regrid(dgf_forest* f, const std::vector<uint64_t>& old_leaves) {
   const bool carry = f->device >= 0 && f->have_state;
-  if (!carry) return build_device(f);
+  if (!carry) return build_all(f);
   const int d = f->d, n = f->n, N = f->N, M = f->M, nc = f->nc, NW = 1 << d;
   DeviceGuard dg(f->device);
   cudaStreamSynchronize(f->stream);
@@ -2174,6 +2198,7 @@ static dgf_status regrid(dgf_forest* f, const std::vector<uint64_t>& old_leaves)
     f->have_state = false;
     return st;
   }
+  if ((st = build_metric(f))) return st;
   return init_lambda(f);
 }
 
