@@ -77,13 +77,32 @@ def leaf_count(workload):
     return leaves
 
 
+def _curved(workload):
+    """Does some root have cells that are not one parallelepiped repeated?"""
+    d, n = workload["dim"], workload["n_seg"]
+    cells = workload.get("root_cell_nodes")
+    if cells is None:
+        n, nodes = 1, np.asarray(workload["nodes"], float)
+        cells = (nodes[np.asarray(c)] for c in workload["root_corners"])
+    for x in cells:
+        x = np.asarray(x, float).reshape(*[n + 1] * d, d)
+        for a in range(d):
+            e = np.diff(x, axis=a)
+            e0 = e[(0,) * d]
+            if np.abs(e - e0).max() > 1e-12 * np.abs(e0).max():
+                return True
+    return False
+
+
 def footprint_bytes(workload, p, precision=FP32):
     """Device bytes a solve holds while resident, estimated before it is
     built: three stage buffers (for the compensated form two more in FP64
     and u^n split into two FP32 arrays),
     the cell map coefficients and cell sizes in the compute precision and in
-    FP64, the guard traces and modal guard cells, the per-leaf tables and
-    1 MiB for the finer-face operators and scalars."""
+    FP64, the guard traces and modal guard cells, the per-leaf tables, in
+    FP64 with curved blocks the metric at the Gauss points and at the lower
+    face points of every cell, and 1 MiB for the finer-face operators and
+    scalars."""
     d, n = workload["dim"], workload["n_seg"]
     L = leaf_count(workload)
     nc, N = n ** d, p + 1
@@ -94,7 +113,10 @@ def footprint_bytes(workload, p, precision=FP32):
     geo = L * nc * (((1 << d) - 1) * d + 1) * (es + 8)
     faces = L * 2 * d * (d + 2) * n ** (d - 1)
     guard = faces * N ** (d - 1) * es + faces * M * (es + 8)
-    return int(state + geo + guard + L * 2 * d * 40 + (1 << 20))
+    metric = 0
+    if precision == FP64 and _curved(workload):
+        metric = L * nc * ((d * d + 1) * M + d * d * N ** (d - 1)) * 8
+    return int(state + geo + guard + metric + L * 2 * d * 40 + (1 << 20))
 
 
 # solve and initial-value streams take precedence over batch streams
@@ -307,17 +329,18 @@ class Server:
                         state, _ = s.finish(keep_state)
                         results[s.req.rid] = Result(s.req.rid, s.req.arrival, s.admitted, now, steps, s.dof, t,
                                                     -100, s.bytes, state)
-                    for r in pending + queue:
+                    for r in pending + [r for r, _ in queue]:
                         results[r.rid] = Result(r.rid, r.arrival, now, now, 0, 0, 0.0, -101)
                     break
                 while pending and pending[0].arrival <= now:
-                    queue.append(pending.pop(0))
+                    req = pending.pop(0)
+                    queue.append((req, footprint_bytes(req.workload, req.p, req.precision)))
                 # admission: first come first served, by slot count and footprint
                 while queue and len(active) + len(building) < self.max_active:
-                    est = footprint_bytes(queue[0].workload, queue[0].p, queue[0].precision)
+                    req, est = queue[0]
                     if (active or building) and used + est > self.budget:
                         break
-                    req = queue.pop(0)
+                    queue.pop(0)
                     used += est
                     item = [None, req, est, self.clock() - t0]
                     if pool is not None:
