@@ -1204,9 +1204,11 @@ dgf_status init_lambda(dgf_forest* f) {
 // written to a scratch stage buffer, the state is untouched) for every
 // stage kernel that applies to the forest (the cell-pair kernel and
 // k_stage, each with its own persistent grid) and every z-chunk length n,
-// n/2, ..., 1, and keep the fastest pair (median of 3 launches).  Choices
-// so far, by (device, dim, p, n, precision, leaves, all affine): a forest of
-// a shape already timed in this process takes the earlier choice.
+// n/2, ..., 1, and keep the fastest pair (median of 3 launches).  Choices so
+// far, by what decides the times: device, dim, p, n, precision, leaves, kinds
+// of blocks, level-jump treatment, to a factor of two the faces left to the
+// guard pass, and what is pinned; a forest of a shape already timed in this
+// process takes the earlier choice.
 // DGF_ZCHUNK fixes the chunk length, DGF_STAGE_KERNEL=classic|pair the kernel.
 std::mutex g_tune_mutex;
 struct TuneChoice {
@@ -1218,7 +1220,17 @@ std::map<std::vector<long long>, TuneChoice> g_tune_cache;
 dgf_status autotune(dgf_forest* f) {
   f->tuned = true;
   if (f->d != 3 || f->slots <= 0) return DGF_OK;
-  const std::vector<long long> key = {f->device, f->d, f->p, f->n, f->precision, (long long)f->nL, f->all_affine};
+  const bool mixed =
+      !f->all_affine && std::any_of(f->h_affine.begin(), f->h_affine.end(), [](unsigned char a) { return a != 0; });
+  int jumps = 0;
+  for (int64_t faces = f->ntr + f->nfine; faces > 0; faces >>= 1) ++jumps;
+  const char* ks = getenv("DGF_STAGE_KERNEL");
+  const long long pins[3] = {ks ? (ks[0] == 'c' ? 1 : strcmp(ks, "pair5") == 0 ? 2 : 0) : -1,
+                             getenv("DGF_ZCHUNK") ? f->zchunk : -1,
+                             getenv("DGF_STAGE_GRID") ? (long long)grid_env(false) : -1};
+  const std::vector<long long> key = {f->device,     f->d,  f->p,      f->n,  f->precision, (long long)f->nL,
+                                      f->all_affine, mixed, f->mortar, jumps, pins[0],      pins[1],
+                                      pins[2]};
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tune_cache.find(key);
@@ -1234,7 +1246,6 @@ dgf_status autotune(dgf_forest* f) {
   if (!st) st = cuda_check(do_guard(f, guard_args(f, 0, f->gtr.ptr, 1, 1)), "guard");  // every face, for every candidate
   if (st) return st;
   std::vector<int> kernels;
-  const char* ks = getenv("DGF_STAGE_KERNEL");
   // the cell-pair kernel is a candidate only where it applies (distinct
   // slots), its second CTA shape at p = 1; DGF_STAGE_KERNEL=pair|pair5|classic
   // keeps one
