@@ -1203,12 +1203,13 @@ dgf_status init_lambda(dgf_forest* f) {
 // Autotuner for the stage kernel: time one residual evaluation (mode 1,
 // written to a scratch stage buffer, the state is untouched) for every
 // stage kernel that applies to the forest (the cell-pair kernel and
-// k_stage, each with its own persistent grid) and every z-chunk length n,
-// n/2, ..., 1, and keep the fastest pair (median of 3 launches).  Choices so
-// far, by what decides the times: device, dim, p, n, precision, leaves, kinds
-// of blocks, level-jump treatment, to a factor of two the faces left to the
-// guard pass, and what is pinned; a forest of a shape already timed in this
-// process takes the earlier choice.
+// k_stage), its grids and every z-chunk length n, n/2, ..., 1; then the best
+// of each kernel in a whole step with the guard passes that it needs (the
+// cell-pair kernel traces most faces itself, k_stage none), and keep the
+// fastest (medians).  Choices so far, by what decides the times:
+// device, dim, p, n, precision, leaves, kinds of blocks, level-jump treatment,
+// to a factor of two the faces left to the guard pass, and what is pinned; a
+// forest of a shape already timed in this process takes the earlier choice.
 // DGF_ZCHUNK fixes the chunk length, DGF_STAGE_KERNEL=classic|pair the kernel.
 std::mutex g_tune_mutex;
 struct TuneChoice {
@@ -1263,49 +1264,101 @@ dgf_status autotune(dgf_forest* f) {
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
-  int best_z = f->zchunk, best_k = f->kernel;
-  bool best_g = f->grid_items;
-  float best = 1e30f;
+  // median of R launches after a warm-up, into *out
+  auto timed = [&](int R, auto&& launch, float* out) -> cudaError_t {
+    std::vector<float> t(R);
+    for (int r = 0; r <= R; ++r) {
+      cudaEventRecord(a, f->stream);
+      if (cudaError_t e = launch()) return e;
+      cudaEventRecord(b, f->stream);
+      cudaEventSynchronize(b);
+      if (r > 0) cudaEventElapsedTime(&t[r - 1], a, b);
+    }
+    std::sort(t.begin(), t.end());
+    *out = t[R / 2];
+    return cudaSuccess;
+  };
+  auto stage = [&]() { return do_stage(f, stage_args(f, 0, 1, 0.0, 1.0, 1, 0)); };
+  auto take = [&](const TuneChoice& c) {
+    f->kernel = c.kernel;
+    f->slots = f->slots_k[c.kernel];
+    f->zchunk = c.zchunk;
+    f->grid_items = c.grid_items;
+  };
+  const TuneChoice was{f->zchunk, f->kernel, f->grid_items};
+  TuneChoice best = was;
+  cudaError_t e = cudaSuccess;
+  float least = 1e30f;
   for (int kk : kernels) {
-    f->kernel = kk;
-    f->slots = f->slots_k[kk];
+    TuneChoice mine{was.zchunk, kk, was.grid_items};
+    float ms = 1e30f;
     for (int gm : grids)
-    for (int z : zs) {
-      f->zchunk = z;
-      f->grid_items = gm != 0;
-      float t[3];
-      for (int r = 0; r < 4; ++r) {
-        cudaEventRecord(a, f->stream);
-        cudaError_t e = do_stage(f, stage_args(f, 0, 1, 0.0, 1.0, 1, 0));
-        cudaEventRecord(b, f->stream);
-        if (e != cudaSuccess) {
-          cudaEventDestroy(a);
-          cudaEventDestroy(b);
-          return cuda_check(e, "autotune");
+      for (int z : zs) {
+        const TuneChoice c{z, kk, gm != 0};
+        take(c);
+        float t = 0.f;
+        if (!e) e = timed(3, stage, &t);
+        if (!e && t < ms) {
+          ms = t;
+          mine = c;
         }
-        cudaEventSynchronize(b);
-        if (r > 0) cudaEventElapsedTime(&t[r - 1], a, b);  // first launch warms up
       }
-      std::sort(t, t + 3);
-      // k_stage must beat the cell-pair kernel by 2 % to be chosen, so that
-      // timing noise does not flip the choice (the kernels round differently)
-      const float tt = kk == 1 && !kernels.empty() && kernels[0] == 0 ? t[1] * 1.02f : t[1];
-      if (tt < best) {
-        best = tt;
-        best_z = z;
-        best_k = kk;
-        best_g = gm != 0;
+    if (kernels.size() > 1) {
+      // stages alone that take longer than another kernel's whole step (with
+      // a tenth for the events around each): out
+      if (3.f * ms > 1.1f * least) continue;
+      take(mine);
+      // the three stages of a time step, but within the two stage buffers,
+      // with scratch for the CFL minimum and the status, and with the current
+      // CFL minimum as time increment (the increment may still be 0); replayed
+      // as a graph, as a step is, a few at a time where they are short
+      auto whole = [&]() {
+        const double ca[3] = {0.0, 0.75, 1.0 / 3.0};
+        cudaError_t r = cudaSuccess;
+        for (int k = 0; k < 3 && !r; ++k) {
+          RtStage s = stage_args(f, k, k == 1 ? 2 : 1, ca[k], 1.0 - ca[k], 0, k == 2);
+          s.dtp = (const double*)s.lam_bits;
+          s.lam_bits = (unsigned long long*)f->tot.ptr;
+          s.status = (int*)((double*)f->tot.ptr + 1);
+          r = do_guard(f, guard_args(f, k, f->gtr.ptr, 1, kk));
+          if (!r) r = do_stage(f, s);
+        }
+        return r;
+      };
+      cudaGraph_t g = nullptr;
+      cudaGraphExec_t x = nullptr;
+      if (!e) e = cudaStreamBeginCapture(f->stream, cudaStreamCaptureModeThreadLocal);
+      if (!e) {
+        const cudaError_t w = whole();
+        e = cudaStreamEndCapture(f->stream, &g);
+        if (w) e = w;
       }
+      if (!e) e = cudaGraphInstantiate(&x, g, 0);
+      const int reps = std::max(1, std::min(4, (int)(0.05f / ms)));
+      auto steps = [&]() {
+        cudaError_t r = cudaSuccess;
+        for (int i = 0; i < reps && !r; ++i) r = cudaGraphLaunch(x, f->stream);
+        return r;
+      };
+      if (!e) e = timed(3, steps, &ms);
+      ms /= (float)reps;
+      if (x) cudaGraphExecDestroy(x);
+      if (g) cudaGraphDestroy(g);
+    }
+    // k_stage must beat the cell-pair kernel by 2 % to be chosen, so that
+    // timing noise does not flip the choice (the kernels round differently)
+    if (kk == 1 && kernels[0] == 0) ms *= 1.02f;
+    if (ms < least) {
+      least = ms;
+      best = mine;
     }
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
-  f->zchunk = best_z;
-  f->kernel = best_k;
-  f->grid_items = best_g;
-  f->slots = f->slots_k[best_k];
+  take(e ? was : best);
+  if (e) return cuda_check(e, "autotune");
   std::lock_guard<std::mutex> lock(g_tune_mutex);
-  g_tune_cache[key] = {best_z, best_k, best_g};
+  g_tune_cache[key] = best;
   return DGF_OK;
 }
 

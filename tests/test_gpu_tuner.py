@@ -1,9 +1,18 @@
-"""What the first time step of a forest picks: stage kernel, chunk length, grid."""
+"""What the first time step of a forest picks: stage kernel, chunk length, grid.
+
+The cell-pair kernel traces most faces itself and the layer-sweep kernel leaves
+them to the guard pass, so the picked kernel is the one with the shorter whole
+step, which stage times alone do not tell."""
+import statistics
+import time
+
 import pytest
 
 import workloads as W
 
 pytestmark = pytest.mark.gpu
+
+KERNELS = ("pair", "pair5", "classic")
 
 
 @pytest.fixture(scope="module")
@@ -13,11 +22,56 @@ def dgf():
     return pkg
 
 
+def curved(B):
+    return W.lattice_forest(3, B, 1.0, 8, jitter=0.1, rotate_roots=True, seed=1)
+
+
+def jumps():
+    w = W.lattice_forest(3, 4, 1.0, 8)
+    w["refine"] = [[(r, 1, (0, 0, 0)) for r in (21, 22, 25, 26, 37, 38, 41, 42)]]
+    return w
+
+
 def forest(dgf, w, p, mode):
     f = dgf.Forest.from_workload(w, p=p, precision=dgf.FP32, cfl=0.05, nonconforming=mode)
     f.project(W.smooth_state)
     f.run(5)
     return f
+
+
+def step_us(f, steps=30):
+    t0 = time.perf_counter()
+    f.run(steps)  # reads the time at the end: waits
+    return (time.perf_counter() - t0) / steps * 1e6
+
+
+@pytest.mark.parametrize("name,make,p,mode", [
+    ("71 leaves", lambda: W.jitter3d_forest(seed=0), 2, "paper"),
+    ("71 leaves", lambda: W.jitter3d_forest(seed=0), 2, "mortar"),
+    ("one level, curved", lambda: curved(4), 1, "paper"),
+    ("one level, curved", lambda: curved(4), 2, "paper"),
+    ("level jumps, affine", jumps, 1, "paper"),
+])
+def test_picked_kernel_has_the_shortest_step(dgf, name, make, p, mode, monkeypatch):
+    """Every kernel pinned in turn beside the free choice, their steps timed
+    alternately; the 2 % that the layer-sweep kernel has to win by and 6 % for
+    host timing."""
+    w = make()
+    fs = {}
+    for k in KERNELS if p == 1 else ("pair", "classic"):
+        monkeypatch.setenv("DGF_STAGE_KERNEL", k)
+        fs[k] = forest(dgf, w, p, mode)
+        assert fs[k].tuning()["stage_kernel"] == k
+    monkeypatch.delenv("DGF_STAGE_KERNEL")
+    free = forest(dgf, w, p, mode)
+    t = {k: [] for k in (*fs, "free")}
+    for _ in range(15):
+        for k, f in (*fs.items(), ("free", free)):
+            t[k].append(step_us(f))
+    med = {k: statistics.median(v) for k, v in t.items()}
+    assert med["free"] <= 1.08 * min(med.values()), (name, free.tuning(), med)
+    for f in (*fs.values(), free):
+        f.close()
 
 
 def test_choice_does_not_outlive_a_pin(dgf, monkeypatch):
