@@ -277,7 +277,8 @@ dgf_status dgf_tuning(const dgf_forest* f, int32_t* zchunk, int32_t* resident_ct
 /* Which stage kernel the forest's time step launches (host value, no sync):
  * 0 = the cell-pair FP32 kernel (3D forests of 8^3-cell blocks at p = 1..3
  * in plain FP32: f32x2 arithmetic on cell pairs, TMA-staged layers, traces
- * read from the neighbours; four CTAs per SM at p = 1), 1 = the general
+ * read from the neighbours; four CTAs per SM at p = 1; densities below
+ * 1.2e-38, subnormal in FP32, count as zero), 1 = the general
  * layer-sweep kernel, 2 = the cell-pair kernel in its second CTA shape
  * (p = 1 only; affine forests: five CTAs per SM, more warps with fewer
  * registers).  The first dgf_rk_step of a 3D forest times every kernel that

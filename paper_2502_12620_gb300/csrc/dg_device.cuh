@@ -427,10 +427,16 @@ struct GuardArgs {
 #ifndef DGF_STAGE_MINB_F32_P1
 #define DGF_STAGE_MINB_F32_P1 4
 #endif
+// FP64 takes 256 threads: two warps a scheduler keep its pipe busy, nothing is
+// spilled.  Us a step with 512 threads and with 256, 8^3-cell blocks: 3D p = 0,
+// 512 affine blocks 1621 -> 1602, 216 curved 760 -> 749; 3D p = 1, 64 affine
+// 672 -> 667, 71 curved 743 -> 741, 512 affine 4652 -> 4681, 216 curved 2249 ->
+// 2307 (512 threads ahead by 0.6 and 2.6 %); 2D p = 1, 256 blocks 131 -> 127,
+// 1600 blocks 650 -> 630.
 template <int P, typename Real>
 struct StageCfg {
   static constexpr int NT = sizeof(Real) == 4 ? (P <= 1 ? DGF_STAGE_NT_F32_P1 : P <= 2 ? DGF_STAGE_NT_F32 : 512)
-                                              : 256;  // FP64: two warps a scheduler keep the pipe busy, no spills
+                                              : 256;
   static constexpr int MINB = sizeof(Real) == 4 ? (P <= 1 ? DGF_STAGE_MINB_F32_P1 : P <= 2 ? 2 : 1) : 1;
 };
 
