@@ -207,7 +207,8 @@ dgf_status dgf_quad_points(const dgf_forest* f, double* xyz);
 
 /* Number of state values (leaves * nv * M * n^d). */
 dgf_status dgf_state_size(const dgf_forest* f, int64_t* n_values);
-/* Copy in / out the modal state (layout above; forest element type). */
+/* Copy in / out the modal state (layout above; forest element type).  A device
+ * buffer whose cudaMalloc allocation ends before the state does: DGF_EINVAL. */
 dgf_status dgf_set_state(dgf_forest* f, const void* src, int is_device);
 dgf_status dgf_get_state(dgf_forest* f, void* dst, int is_device);
 /* Set the state from FP64 point values [leaf][cell][q][var] at the volume

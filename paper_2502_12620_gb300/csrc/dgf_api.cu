@@ -7,6 +7,7 @@
 //   k_dt -> 3 x { k_guard (guard traces, Sec. 3.5) ; k_stage (residual +
 //   inverse mass + stage combination, CFL minimum on the last stage) },
 // captured once into a CUDA graph and replayed.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1173,11 +1174,34 @@ bool on_device(const void* p, int device) {
   return (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) && a.device == device;
 }
 
-// A caller's buffer that a kernel may read or write in place of a copy: memory
-// of the forest's device, aligned to its elements.  Anything else a copy can
-// reach (host memory, another device's, unaligned) keeps the staged copy.
-bool kernel_reaches(const dgf_forest* f, const void* p, int is_device, size_t elem) {
-  return is_device && (uintptr_t)p % elem == 0 && on_device(p, f->device);
+template <typename Fn>
+Fn* driver_fn(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &found);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Fn*)p : nullptr;
+}
+
+// How a caller's buffer is reached.  kKernel: memory of the forest's device,
+// aligned to its elements and with all the bytes in one allocation, which a
+// kernel may read or write in place of a copy.  kShort: an allocation of
+// cudaMalloc that ends before the buffer does (a copy would be refused, a
+// kernel would fault).  kCopy: anything else that a copy can reach (host memory,
+// another device's, unaligned, mapped piece by piece) keeps the staged copy.
+enum class Reach { kKernel, kCopy, kShort };
+Reach reach(const dgf_forest* f, const void* p, int is_device, size_t elem, size_t bytes) {
+  if (!is_device || (uintptr_t)p % elem != 0 || !on_device(p, f->device)) return Reach::kCopy;
+  static const auto range = driver_fn<CUresult(CUdeviceptr*, size_t*, CUdeviceptr)>("cuMemGetAddressRange");
+  static const auto attribute = driver_fn<CUresult(void*, CUpointer_attribute, CUdeviceptr)>("cuPointerGetAttribute");
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range || range(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return Reach::kCopy;
+  if ((CUdeviceptr)p - base + bytes <= size) return Reach::kKernel;
+  unsigned long long whole = 0;  // one cudaMalloc, not mapped piece by piece
+  const bool known = attribute && attribute(&whole, CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE, (CUdeviceptr)p) ==
+                                      CUDA_SUCCESS;
+  return known && whole ? Reach::kShort : Reach::kCopy;
 }
 
 // compute-precision buffer -> state-precision buffer (compensated form: FP32 -> FP64)
@@ -1737,7 +1761,9 @@ dgf_status dgf_set_state(dgf_forest* f, const void* src, int is_device) {
   const size_t bytes = (size_t)f->nL * f->nv * f->M * f->nc * f->sesize;
   dgf_status st;
   RtMisc r = misc_args(f, 0);
-  if (kernel_reaches(f, src, is_device, f->sesize)) {
+  const Reach way = reach(f, src, is_device, f->sesize, bytes);
+  if (way == Reach::kShort) return fail(DGF_EINVAL, "set_state: the source is shorter than the state");
+  if (way == Reach::kKernel) {
     r.U = src;
   } else {
     void* tmp = f->comp ? f->U64[1 - f->cur].ptr : f->U[1].ptr;  // free between time steps
@@ -1764,7 +1790,9 @@ dgf_status dgf_get_state(dgf_forest* f, void* dst, int is_device) {
   if (!f->have_state) return fail(DGF_ESTATE, "no state set");
   DeviceGuard dg(f->device);
   const size_t bytes = (size_t)f->nL * f->nv * f->M * f->nc * f->sesize;
-  if (kernel_reaches(f, dst, is_device, f->sesize)) {
+  const Reach way = reach(f, dst, is_device, f->sesize, bytes);
+  if (way == Reach::kShort) return fail(DGF_EINVAL, "get_state: the destination is shorter than the state");
+  if (way == Reach::kKernel) {
     dgf_status st = cuda_check(do_convert(f, state_ptr(f), dst, (size_t)f->nL, f->nc, 0, state_f64(f)), "to modal");
     return st ? st : cuda_check(cudaStreamSynchronize(f->stream), "get_state");
   }
