@@ -51,7 +51,8 @@ HBM_FALLBACK = 6800.0
 # proportional to the leaves: 387.0 MB there, the algorithmic 377.5 MB); the
 # 512-leaf cube at p = 1 fits L2, so no figure is scaled to the 16^3 cube at
 # p = 1.
-STAGE_TRAFFIC_BYTES = {("cube16p2", "pair"): 8 * 387.0e6}
+STAGE_TRAFFIC_BYTES = {("jitter3d", "classic"): 42.6e6, ("jitter3d", "pair"): 36.5e6,
+                       ("cube16p2", "pair"): 8 * 387.0e6}
 TRAFFIC_HOW = "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch, cold L2, mean of the 3 stages of a step"
 
 
