@@ -34,6 +34,14 @@ static Tab<N, Real> make_tab(const RtTables& r) {
   return t;
 }
 
+// SMs of the current device (152 on a whole GB300)
+static inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 152;
+  return n;
+}
+
 // Rows of a 2D block that one stage work item sweeps: the whole block, or a
 // quarter of it when that fills the SMs better.  An item costs its rows plus
 // about 1.5 rows (start-up and the slab's second edge faces), and the SM is
@@ -46,10 +54,11 @@ constexpr int slab_rows_2d() {
 }
 template <int NS>
 static bool use_slabs_2d(int nL) {
-  constexpr int YS = slab_rows_2d<NS>(), SMS = 152;
+  constexpr int YS = slab_rows_2d<NS>();
   if (YS == NS) return false;
-  const double whole = (double)((nL + SMS - 1) / SMS) * (NS + 1.5);
-  const double slabs = (double)(((long long)nL * (NS / YS) + SMS - 1) / SMS) * (YS + 1.5);
+  const int sms = sm_count();
+  const double whole = (double)((nL + sms - 1) / sms) * (NS + 1.5);
+  const double slabs = (double)(((long long)nL * (NS / YS) + sms - 1) / sms) * (YS + 1.5);
   return slabs < whole;
 }
 
@@ -267,7 +276,7 @@ static cudaError_t stage_p(const RtStage& r, cudaStream_t s) {
 
 // Guard cells of finer faces: a block each while all of them fit the GPU at
 // once (eight 256-thread blocks an SM), a warp each beyond two such rounds.
-static inline bool fine_by_warps(const RtGuard& r, int nt) { return (long long)r.nfine * nt > 2 * 8 * 152; }
+static inline bool fine_by_warps(const RtGuard& r, int nt) { return (long long)r.nfine * nt > 2 * 8 * sm_count(); }
 template <int D>
 static int fine_blocks(const RtGuard& r) {
   const int nt = D == 3 ? r.n * r.n : r.n;
@@ -372,7 +381,7 @@ static cudaError_t cfl_p(const RtMisc& r, cudaStream_t s) {
   const int nc = D == 3 ? r.n * r.n * r.n : r.n * r.n;
   const size_t total = (size_t)r.nL * nc * ipow(P + 1, D);
   const int th = 256;
-  const size_t ctas = (total + th - 1) / th, most = 152 * 8;
+  const size_t ctas = (total + th - 1) / th, most = (size_t)sm_count() * 8;
   k_cfl<D, P, Real><<<(unsigned)(ctas < most ? ctas : most), th, 0, s>>>(
       r.nL, r.n, (const Real*)r.U, (const Real*)r.hcell, (Real)r.gamma, r.lam_bits, r.status);
   return cudaGetLastError();
