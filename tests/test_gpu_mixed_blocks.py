@@ -57,11 +57,12 @@ def test_mixed_forest_matches_oracle(dgf, p, mode, monkeypatch):
 @pytest.mark.parametrize("mode", ["paper", "mortar"])
 @pytest.mark.parametrize("p", [1, 2, 3])
 def test_mixed_forest_chunks_and_grids_change_no_bit(dgf, p, mode, monkeypatch):
-    """71 leaves: up to 568 items on at most 456 resident CTAs at p = 1 and
-    152 at p = 2, 3.  One CTA per whole block is the tiling in which no CTA
-    meets a second item."""
-    w = mixed_forest((4, 4, 4))
-    U = W.random_modal_state(71, 3, 8, p, seed=2).astype(np.float32)
+    """157 leaves on at most 456 resident CTAs at p = 1, 71 on 152 at p = 2, 3:
+    more items than CTAs from three-layer chunks down.  One CTA per whole block
+    is the tiling in which no CTA meets a second item.  At p = 1 both CTA
+    shapes."""
+    w = mixed_forest((6, 5, 5) if p == 1 else (4, 4, 4))
+    U = W.random_modal_state(157 if p == 1 else 71, 3, 8, p, seed=2).astype(np.float32)
 
     def result():
         f = dgf.Forest.from_workload(w, p=p, precision=dgf.FP32, cfl=0.2, nonconforming=mode)
@@ -77,12 +78,14 @@ def test_mixed_forest_chunks_and_grids_change_no_bit(dgf, p, mode, monkeypatch):
     monkeypatch.setenv("DGF_ZCHUNK", "8")
     monkeypatch.setenv("DGF_STAGE_GRID", "items")
     R0, U0 = result()
-    for z in (8, 4, 3, 2, 1):
-        for grid in ("persistent", "items"):
-            monkeypatch.setenv("DGF_ZCHUNK", str(z))
-            monkeypatch.setenv("DGF_STAGE_GRID", grid)
-            R, U1 = result()
-            assert np.array_equal(R, R0) and np.array_equal(U1, U0), (z, grid)
+    for kernel in ("pair", "pair5") if p == 1 else ("pair",):
+        monkeypatch.setenv("DGF_STAGE_KERNEL", kernel)
+        for z in (8, 4, 3, 2, 1):
+            for grid in ("persistent", "items"):
+                monkeypatch.setenv("DGF_ZCHUNK", str(z))
+                monkeypatch.setenv("DGF_STAGE_GRID", grid)
+                R, U1 = result()
+                assert np.array_equal(R, R0) and np.array_equal(U1, U0), (kernel, z, grid)
     # tuned freely: every tiling is timed on the way; whichever kernel is taken
     # (each is within TOL of the oracle)
     for k in ("DGF_STAGE_KERNEL", "DGF_ZCHUNK", "DGF_STAGE_GRID"):
